@@ -190,10 +190,33 @@ tucker_status launch_loss_grad(Ctx *c, const float *const *U, const float *G, do
     TK_CUDA(dev_alloc(c, &c->adj_Y, (size_t)ymax));
     TK_CUDA(dev_alloc(c, &c->adj_Q, (size_t)(I1 * P1)));
     TK_CUDA(dev_alloc(c, &c->adj_Gn, (size_t)PR));
+    int64_t packed = 0;
+    for (int m = 0; m < N; ++m) packed += c->dims[m] * tile_layout(c->ranks[m]).row();
+    TK_CUDA(dev_alloc(c, &c->adj_U, (size_t)packed));
     TK_CUDA(dev_alloc(c, &c->adj_part, (size_t)kAdjRedBlocks));
     TK_CUDA(dev_alloc(c, &c->adj_gpart, (size_t)(64 * PR)));
     TK_CUDA(cudaStreamSynchronize(s));
     c->astream = 0;
+  }
+  // (0) the factors as the TTMc reads them: copies in tile_layout, unless the caller's are that already
+  const float *Up[kMaxOrder];
+  {
+    TilePack pk{};
+    int copies = 0;
+    float *at = c->adj_U;
+    for (int m = 0; m < N; ++m) {
+      Up[m] = U[m];
+      const int64_t n = c->dims[m] * tile_layout(c->ranks[m]).row();
+      if (!tile_plain(c->ranks[m]) || reinterpret_cast<uintptr_t>(U[m]) % 16 != 0) {
+        pk.in[copies] = U[m];
+        pk.out[copies] = at;
+        pk.I[copies] = c->dims[m];
+        pk.R[copies++] = c->ranks[m];
+        Up[m] = at;
+      }
+      at += n;
+    }
+    if (copies) launch_tile_pack(pk, copies, s);
   }
   // (1) Q = U_1 G_(1)
   adj_q_kernel<<<blocks_for(I1 * P1), 256, 0, s>>>(U[0], G, I1, R1, P1, c->adj_Q);
@@ -225,7 +248,7 @@ tucker_status launch_loss_grad(Ctx *c, const float *const *U, const float *G, do
       ::tk::count_launch();
       en = c->adj_en;
     }
-    tucker_status st = launch_ttmc_ex(c, n, c->adj_Y, en, U, s);
+    tucker_status st = launch_ttmc_ex(c, n, c->adj_Y, en, Up, s);
     if (st != TUCKER_OK) return st;
     Unfold uf{};
     uf.N = N;

@@ -36,18 +36,34 @@ void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 uint64_t launches_so_far() { return g_launches.load(std::memory_order_relaxed); }
 void count_launches(int64_t delta) { g_launches.fetch_add((uint64_t)delta, std::memory_order_relaxed); }
 
-__global__ void f64_to_f32_kernel(const double *in, int64_t n, float *out32, __nv_bfloat16 *out16) {
+// FP32 copy of a factor in tile_layout (rows of `row` floats, a power of two, the chunks'
+// padding zero), and its plain BF16 copy; with a BF16 copy the FP32 one holds the same values.
+__global__ void f64_to_f32_kernel(const double *in, int64_t I, int R, TileLayout l, float *out32,
+                                  __nv_bfloat16 *out16) {
+  const int row = l.row(), sh = 31 - __clz(row);
+  const int64_t n = I << sh;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double v = in[i];
-    out32[i] = __double2float_rn(v);
-    if (out16) out16[i] = __double2bfloat16(v);
+    const int r = l.rank((int)(i & (row - 1)), R);
+    float f = 0.f;
+    if (r >= 0) {
+      const int64_t src = (i >> sh) * R + r;
+      const double v = in[src];
+      f = __double2float_rn(v);
+      if (out16) {
+        const __nv_bfloat16 h = __double2bfloat16(v);
+        out16[src] = h;
+        f = __bfloat162float(h);
+      }
+    }
+    out32[i] = f;
   }
 }
 
 void refresh_factor_copies(Ctx *c, int m, cudaStream_t s) {
-  const int64_t n = c->dims[m] * c->ranks[m];
+  const TileLayout l = tile_layout(c->ranks[m]);
+  const int64_t n = c->dims[m] * l.row();
   const unsigned b = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 4096));
-  f64_to_f32_kernel<<<b, 256, 0, s>>>(c->U64[m], n, c->U32[m], c->U16[m]);
+  f64_to_f32_kernel<<<b, 256, 0, s>>>(c->U64[m], c->dims[m], c->ranks[m], l, c->U32[m], c->U16[m]);
   ::tk::count_launch();
 }
 
@@ -213,7 +229,7 @@ static tucker_status init_impl(Ctx *c, const uint32_t *coords, const float *vals
   for (int m = 0; m < N; ++m) {
     const size_t n = (size_t)(c->dims[m] * c->ranks[m]);
     TK_CUDA(dev_alloc(c, &c->U64[m], n));
-    TK_CUDA(dev_alloc(c, &c->U32[m], n));
+    TK_CUDA(dev_alloc(c, &c->U32[m], (size_t)(c->dims[m] * tile_layout(c->ranks[m]).row())));
     if (c->flags & TUCKER_F_BF16_FACTORS) TK_CUDA(dev_alloc(c, &c->U16[m], n));
   }
   if (U0) {

@@ -108,7 +108,8 @@ struct Ctx {
   ModeCopy mode[kMaxOrder];
 
   double *U64[kMaxOrder] = {};        // FP64 master factors
-  float *U32[kMaxOrder] = {};         // FP32 copies read by the TTMc
+  float *U32[kMaxOrder] = {};         // FP32 copies read by the TTMc, in tile_layout (of the BF16 values with
+                                      // TUCKER_F_BF16_FACTORS)
   __nv_bfloat16 *U16[kMaxOrder] = {}; // BF16 copies (TUCKER_F_BF16_FACTORS)
   // TMA descriptors of the BF16 copies (rows of one factor, one row per box) for the row
   // gathers of the pipelined BF16 TTMc; tm16_ok[m] false where none could be made
@@ -138,6 +139,7 @@ struct Ctx {
   float *adj_Y = nullptr;      // TTMc of the residual tensor (max I_n * P_n)
   float *adj_Q = nullptr;      // U_1 G_(1) (I_1 x P_1)
   float *adj_Gn = nullptr;     // one unfolding of G (prod R)
+  float *adj_U = nullptr;      // the caller's factors in tile_layout, one after another
   double *adj_part = nullptr;  // loss partials
   float *adj_gpart = nullptr;  // split-K partials of dL/dG
   bool G_valid = false;
@@ -224,6 +226,62 @@ void fill_iota_ones(uint32_t *iota, float *ones, int64_t n, cudaStream_t s);
 // TTMc of mode `mode` with values `val` (in that mode's sorted order) and FP32 factors
 // Uf[m] (indexed by mode; Uf[mode] unused) instead of the context's own.
 tucker_status launch_ttmc_ex(Ctx *c, int mode, float *Y, const float *val, const float *const *Uf, cudaStream_t s);
+
+// ---- K-b, tiled form (ttmc_tile.cuh): FP32, any order and ranks
+// A factor copy for it: the R ranks in n = 1, 2, 4 or 8 chunks of at most T <= 8, of which
+// the first four of every chunk come first (chunk c in floats 4c .. 4c + 3), then what is
+// left of every chunk (floats 4(n + c) ..), zero where there is nothing; a row is a power of
+// two of floats.  Chunks of eight hold the ranks that stand there in a plain row (`jump`: ranks
+// skipped between their halves); smaller ones T consecutive ranks.
+struct TileLayout {
+  int n, T, jump;
+  __host__ __device__ constexpr int row() const { return T <= 4 ? 4 * n : 8 * n; }
+  // place in the row of rank r
+  __host__ __device__ constexpr int pos(int r) const {
+    return T == 8 ? r : r % T < 4 ? r / T * 4 + r % T : 4 * (n + r / T) + r % T - 4;
+  }
+  // rank at place q of the row, or -1 (for a rank below R)
+  __host__ __device__ constexpr int rank(int q, int R) const {
+    if (T == 8) return q < R ? q : -1;
+    const int c = q / 4 % n, o = q / (4 * n) * 4 + q % 4, r = c * T + o;
+    return o < T && r < R ? r : -1;
+  }
+};
+__host__ __device__ constexpr TileLayout tile_layout(int R) {
+  TileLayout l{};
+  l.n = 1;
+  while ((R + l.n - 1) / l.n > 8) l.n *= 2;
+  l.T = (R + l.n - 1) / l.n;
+  l.jump = l.T == 8 ? 4 * l.n - 4 : 0;
+  return l;
+}
+inline bool tile_plain(int R) { return tile_layout(R).row() == R; }  // the copy is the plain matrix
+struct TileCall {
+  int nother;                       // remaining modes, ascending:
+  const uint32_t *idx[kMaxOrder];   //   sorted coordinates
+  const float *U[kMaxOrder];        //   factor copies in tile_layout, 16-byte aligned
+  int R[kMaxOrder];
+  const float *val;                 // value of sorted position e: val[vsrc[e]], or val[e] with vsrc null
+  const uint32_t *vsrc;
+  const uint32_t *sptr, *sid;
+  uint32_t S;
+  const uint32_t *unit_e0, *unit_k0;
+  const int32_t *unit_slot;
+  int64_t n_units;
+  uint32_t Z;
+  float *Y, *carry;
+  int64_t P;
+  double slice_len;                 // nonzeros per non-empty slice on average
+  int num_sms;
+};
+cudaError_t launch_ttmc_tile(const TileCall &c, cudaStream_t s);
+struct TilePack {  // plain row-major factors to copies in tile_layout
+  const float *in[kMaxOrder];
+  float *out[kMaxOrder];
+  int64_t I[kMaxOrder];
+  int R[kMaxOrder];
+};
+void launch_tile_pack(const TilePack &p, int modes, cudaStream_t s);
 
 // ---- K-c: QRP (qrp.cu)
 size_t qrp_work_bytes(int64_t m, int64_t n, int k, int nb);

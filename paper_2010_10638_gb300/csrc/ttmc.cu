@@ -120,9 +120,8 @@ __device__ __forceinline__ void lds(const float *p, float (&v)[T]) {
   }
 }
 
-// NL = number of left modes (0, 1 or 2); PL = product of their ranks; RB = rank of the
-// last remaining mode.  Requires RB % 4 == 0, and for NL == 2 the second left rank % 4 == 0.
-template <int NL, int PL, int RB, int TA, int TB, typename FT>
+// Order 3: PL, RB = ranks of the two remaining modes, multiples of 4 (TUCKER_F_UNPIPELINED).
+template <int PL, int RB, int TA, int TB>
 __global__ void __launch_bounds__(kTtmcWarps * 32) ttmc_fast_kernel(const TtmcParams p) {
   constexpr int G = (PL / TA) * (RB / TB);  // lanes per group
   constexpr int NG = 32 / G;                // groups per warp
@@ -135,8 +134,8 @@ __global__ void __launch_bounds__(kTtmcWarps * 32) ttmc_fast_kernel(const TtmcPa
   const int64_t u = (int64_t)blockIdx.x * kTtmcWarps + w;
   if (u >= p.n_units) return;
 
-  const FT *UB = static_cast<const FT *>(p.U[NL]);
-  const uint32_t *idxB = p.idx[NL];
+  const float *U0 = static_cast<const float *>(p.U[0]);
+  const float *UB = static_cast<const float *>(p.U[1]);
   uint32_t e = __ldg(p.unit_e0 + u);
   const uint32_t e_end = (u + 1 < p.n_units) ? __ldg(p.unit_e0 + u + 1) : p.Z;
   uint32_t kb = __ldg(p.unit_k0 + u);
@@ -155,56 +154,31 @@ __global__ void __launch_bounds__(kTtmcWarps * 32) ttmc_fast_kernel(const TtmcPa
     const TileSlices ts = tile_slices(p.sptr, p.S, kb, e, nt, lane);
 
     float x = 0.f;
-    uint32_t i0 = 0, i1 = 0, ib = 0;
+    uint32_t i0 = 0, ib = 0;
     if (lane < nt) {
       x = __ldg(p.val + e + lane);
-      ib = __ldg(idxB + e + lane);
-      if constexpr (NL >= 1) i0 = __ldg(p.idx[0] + e + lane);
-      if constexpr (NL >= 2) i1 = __ldg(p.idx[1] + e + lane);
+      ib = __ldg(p.idx[1] + e + lane);
+      i0 = __ldg(p.idx[0] + e + lane);
     }
     __syncwarp();
     // ---- stage x * kron(left rows) and the last-mode rows
-    if constexpr (NL == 0) {
-      xa[lane] = x;
-    } else if constexpr (NL == 1) {
-      const FT *U0 = static_cast<const FT *>(p.U[0]);
 #pragma unroll
-      for (int it = lane; it < 32 * (PL / 4); it += 32) {
-        const int t = it / (PL / 4), c = (it % (PL / 4)) * 4;
-        const float xt = __shfl_sync(kFull, x, t);
-        const uint32_t r = __shfl_sync(kFull, i0, t);
-        float4 v = Ld<FT>::v4(U0 + (size_t)r * PL, c);
-        v.x *= xt;
-        v.y *= xt;
-        v.z *= xt;
-        v.w *= xt;
-        *reinterpret_cast<float4 *>(xa + t * PL + c) = v;
-      }
-    } else {
-      const FT *U0 = static_cast<const FT *>(p.U[0]);
-      const FT *U1 = static_cast<const FT *>(p.U[1]);
-      const int R1 = p.R[1], R0 = p.R[0];
-#pragma unroll 4
-      for (int it = lane; it < 32 * (PL / 4); it += 32) {
-        const int t = it / (PL / 4), c = (it % (PL / 4)) * 4;
-        const float xt = __shfl_sync(kFull, x, t);
-        const uint32_t r0 = __shfl_sync(kFull, i0, t);
-        const uint32_t r1 = __shfl_sync(kFull, i1, t);
-        const int a0 = c / R1, a1 = c - a0 * R1;
-        const float s0 = xt * Ld<FT>::s(U0 + (size_t)r0 * R0, a0);
-        float4 v = Ld<FT>::v4(U1 + (size_t)r1 * R1, a1);
-        v.x *= s0;
-        v.y *= s0;
-        v.z *= s0;
-        v.w *= s0;
-        *reinterpret_cast<float4 *>(xa + t * PL + c) = v;
-      }
+    for (int it = lane; it < 32 * (PL / 4); it += 32) {
+      const int t = it / (PL / 4), c = (it % (PL / 4)) * 4;
+      const float xt = __shfl_sync(kFull, x, t);
+      const uint32_t r = __shfl_sync(kFull, i0, t);
+      float4 v = Ld<float>::v4(U0 + (size_t)r * PL, c);
+      v.x *= xt;
+      v.y *= xt;
+      v.z *= xt;
+      v.w *= xt;
+      *reinterpret_cast<float4 *>(xa + t * PL + c) = v;
     }
 #pragma unroll
     for (int it = lane; it < 32 * (RB / 4); it += 32) {
       const int t = it / (RB / 4), c = (it % (RB / 4)) * 4;
       const uint32_t r = __shfl_sync(kFull, ib, t);
-      *reinterpret_cast<float4 *>(bb + t * RB + c) = Ld<FT>::v4(UB + (size_t)r * RB, c);
+      *reinterpret_cast<float4 *>(bb + t * RB + c) = Ld<float>::v4(UB + (size_t)r * RB, c);
     }
     __syncwarp();
 
@@ -1360,84 +1334,6 @@ __global__ void __launch_bounds__(kTmaWarps * 32) ttmc_bf16_tma_kernel(const Ttm
   }
 }
 
-// Any shape: each lane owns CPL columns of a block of 32*CPL columns (grid.y), and
-// forms its Kronecker entries directly from the factor rows (cached loads).
-template <int CPL, typename FT>
-__global__ void __launch_bounds__(kTtmcWarps * 32) ttmc_generic_kernel(const TtmcParams p) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t u = (int64_t)blockIdx.x * kTtmcWarps + w;
-  if (u >= p.n_units) return;
-  const int nother = p.nother;
-  // column decode
-  int rr[CPL][kMaxOrder];
-  bool own[CPL];
-  int64_t col[CPL];
-#pragma unroll
-  for (int s = 0; s < CPL; ++s) {
-    col[s] = (int64_t)blockIdx.y * 32 * CPL + lane + 32 * s;
-    own[s] = col[s] < p.P;
-    int64_t cc = own[s] ? col[s] : 0;
-    for (int t = kMaxOrder - 1; t >= 0; --t) {
-      if (t < nother) {
-        rr[s][t] = (int)(cc % p.R[t]);
-        cc /= p.R[t];
-      } else {
-        rr[s][t] = 0;
-      }
-    }
-  }
-  uint32_t e = __ldg(p.unit_e0 + u);
-  const uint32_t e_end = (u + 1 < p.n_units) ? __ldg(p.unit_e0 + u + 1) : p.Z;
-  uint32_t kb = __ldg(p.unit_k0 + u);
-  const int slot = __ldg(p.unit_slot + u);
-  float acc[CPL];
-#pragma unroll
-  for (int s = 0; s < CPL; ++s) acc[s] = 0.f;
-  while (e < e_end) {
-    const int nt = (int)min(32u, e_end - e);
-    const TileSlices ts = tile_slices(p.sptr, p.S, kb, e, nt, lane);
-    float x = 0.f;
-    uint32_t id[kMaxOrder];
-#pragma unroll
-    for (int t = 0; t < kMaxOrder; ++t) id[t] = 0;
-    if (lane < nt) {
-      x = __ldg(p.val + e + lane);
-      for (int t = 0; t < nother; ++t) id[t] = __ldg(p.idx[t] + e + lane);
-    }
-    uint32_t segs = ts.starts | 1u;
-    while (segs) {
-      const int p0 = __ffs(segs) - 1;
-      segs &= segs - 1u;
-      const int p1 = segs ? (__ffs(segs) - 1) : nt;
-      for (int q = p0; q < p1; ++q) {
-        const float xq = __shfl_sync(kFull, x, q);
-        uint32_t iq[kMaxOrder];
-#pragma unroll
-        for (int t = 0; t < kMaxOrder; ++t) iq[t] = __shfl_sync(kFull, id[t], q);
-#pragma unroll
-        for (int s = 0; s < CPL; ++s) {
-          float v = xq;
-          for (int t = 0; t < nother; ++t)
-            v *= Ld<FT>::s(static_cast<const FT *>(p.U[t]) + (size_t)iq[t] * p.R[t], rr[s][t]);
-          acc[s] += v;
-        }
-      }
-      const bool flush = (p1 < nt) || ts.end_is_start || (e + (uint32_t)nt == e_end);
-      if (flush) {
-        const uint32_t kseg = __shfl_sync(kFull, ts.kp, p0);
-        float *dst = (slot >= 0) ? p.carry + (size_t)slot * p.P : p.Y + (size_t)__ldg(p.sid + kseg) * p.P;
-#pragma unroll
-        for (int s = 0; s < CPL; ++s) {
-          if (own[s]) dst[col[s]] = acc[s];
-          acc[s] = 0.f;
-        }
-      }
-    }
-    kb = ts.kb_next;
-    e += (uint32_t)nt;
-  }
-}
-
 // Rows of slices split over several units: block (l, c) sums the partial rows of long
 // slice l for columns [32c, 32c + 32).  Warp w adds the pieces w, w + 8, ... (four loads in
 // flight), then the eight warp sums are added in warp order: a fixed order, so Y is
@@ -1564,10 +1460,10 @@ __global__ void ttmc_zero_rows_kernel(const uint32_t *rows, int64_t n, float *Y,
   }
 }
 
-template <int NL, int PL, int RB, int TA, int TB, typename FT>
+template <int PL, int RB, int TA, int TB>
 static cudaError_t run_fast(const TtmcParams &p, cudaStream_t s) {
   const size_t smem = (size_t)kTtmcWarps * 32 * (PL + RB) * sizeof(float);
-  auto kern = ttmc_fast_kernel<NL, PL, RB, TA, TB, FT>;
+  auto kern = ttmc_fast_kernel<PL, RB, TA, TB>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -1707,45 +1603,20 @@ static bool dispatch_pipe(const TtmcParams &p, cudaStream_t s, cudaError_t *err)
   return false;
 }
 
-template <typename FT>
-static cudaError_t run_generic(const TtmcParams &p, cudaStream_t s) {
-  constexpr int CPL = 4;
-  const unsigned blocks = (unsigned)((p.n_units + kTtmcWarps - 1) / kTtmcWarps);
-  const unsigned cols = (unsigned)((p.P + 32 * CPL - 1) / (32 * CPL));
-  ttmc_generic_kernel<CPL, FT><<<dim3(blocks, cols), kTtmcWarps * 32, 0, s>>>(p);
-  ::tk::count_launch();
-  return cudaGetLastError();
-}
-
-// Shape dispatch.  Returns false when no specialised kernel covers the shape.
-template <typename FT>
+// TUCKER_F_UNPIPELINED: the shapes of the pipelined kernel, without its prefetch.
 static bool dispatch_fast(const TtmcParams &p, cudaStream_t s, cudaError_t *err) {
-  const int no = p.nother;
-  const int RB = p.R[no - 1];
-#define TK_FAST(NL_, PL_, RB_, TA_, TB_)                   \
-  {                                                        \
-    *err = run_fast<NL_, PL_, RB_, TA_, TB_, FT>(p, s);    \
-    return true;                                           \
+  if (p.nother != 2) return false;
+  const int PL = p.R[0], RB = p.R[1];
+#define TK_FAST(PL_, RB_, TA_, TB_)               \
+  if (PL == PL_ && RB == RB_) {                   \
+    *err = run_fast<PL_, RB_, TA_, TB_>(p, s);    \
+    return true;                                  \
   }
-  if (no == 1) {
-    if (RB == 16) TK_FAST(0, 1, 16, 1, 4)
-    if (RB == 32) TK_FAST(0, 1, 32, 1, 4)
-    if (RB == 8) TK_FAST(0, 1, 8, 1, 4)
-  } else if (no == 2) {
-    const int PL = p.R[0];
-    if (PL == 16 && RB == 16) TK_FAST(1, 16, 16, 4, 4)
-    if (PL == 8 && RB == 8) TK_FAST(1, 8, 8, 2, 4)
-    if (PL == 32 && RB == 32) TK_FAST(1, 32, 32, 8, 4)
-    if (PL == 16 && RB == 8) TK_FAST(1, 16, 8, 4, 4)
-    if (PL == 8 && RB == 16) TK_FAST(1, 8, 16, 4, 4)
-  } else if (no == 3) {
-    const int PL = p.R[0] * p.R[1];
-    if (p.R[1] % 4 == 0) {
-      if (PL == 64 && RB == 8) TK_FAST(2, 64, 8, 4, 4)
-      if (PL == 64 && RB == 16) TK_FAST(2, 64, 16, 8, 4)
-      if (PL == 16 && RB == 4) TK_FAST(2, 16, 4, 2, 4)
-    }
-  }
+  TK_FAST(16, 16, 4, 4)
+  TK_FAST(8, 8, 2, 4)
+  TK_FAST(32, 32, 8, 4)
+  TK_FAST(16, 8, 4, 4)
+  TK_FAST(8, 16, 4, 4)
 #undef TK_FAST
   return false;
 }
@@ -1903,8 +1774,37 @@ static tucker_status ttmc_impl(Ctx *c, int mode, float *Y, const float *val, con
       }
       p.sq_part = nullptr;
     }
-    if (!done) done = bf16 ? dispatch_fast<__nv_bfloat16>(p, s, &err) : dispatch_fast<float>(p, s, &err);
-    if (!done) err = bf16 ? run_generic<__nv_bfloat16>(p, s) : run_generic<float>(p, s);
+    if (!done && !bf16 && (c->flags & TUCKER_F_UNPIPELINED)) done = dispatch_fast(p, s, &err);
+    // Every other order and rank: the tiled form (BF16 contexts: FP32 copies of the BF16
+    // factors).  Measured against the kernels it took over, all modes: 600,011 nonzeros, ranks
+    // 12 x 7 x 20 0.118 ms (one thread per column, row entries read per nonzero: 1.036 ms);
+    // 5M nonzeros, ranks 8^4 1.03 ms (4 x 4 tiles, Kronecker rows staged: 2.08 ms); 10M
+    // nonzeros, ranks 10^3 0.90 ms (9.9 ms).
+    if (!done) {
+      TileCall t{};
+      t.nother = mc.nother;
+      for (int q = 0; q < mc.nother; ++q) {
+        const int m = mc.other[q];
+        t.idx[q] = mc.idx[q];
+        t.U[q] = Uf ? Uf[m] : c->U32[m];
+        t.R[q] = c->ranks[m];
+      }
+      t.val = p.val;
+      t.sptr = mc.sptr;
+      t.sid = mc.sid;
+      t.S = (uint32_t)mc.S;
+      t.unit_e0 = mc.unit_e0;
+      t.unit_k0 = mc.unit_k0;
+      t.unit_slot = mc.unit_slot;
+      t.n_units = mc.n_units;
+      t.Z = p.Z;
+      t.Y = Y;
+      t.carry = c->carry;
+      t.P = mc.P;
+      t.slice_len = (double)c->nnz / (double)std::max<int64_t>(mc.S, 1);
+      t.num_sms = c->num_sms;
+      err = launch_ttmc_tile(t, s);
+    }
     TK_CUDA(err);
   }
   if (mc.n_long > 0) {
