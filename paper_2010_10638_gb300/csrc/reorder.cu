@@ -585,22 +585,23 @@ __global__ void unit_fiber_kernel(int64_t n_units, const uint32_t *unit_e0, cons
 
 // units contributed by each non-empty slice k: pieces of a long slice, or 1 for the
 // first slice of a run of short slices (a new run starts at a long slice, after a long
-// slice, and where the slice start crosses into a new multiple of `chunk`).
-__global__ void unit_count_kernel(int64_t S, const uint32_t *sptr, uint32_t chunk, uint32_t *nu, uint32_t *islong) {
+// slice, and where the slice start crosses into a new multiple of `run`).
+__global__ void unit_count_kernel(int64_t S, const uint32_t *sptr, uint32_t chunk, uint32_t run, uint32_t *nu,
+                                  uint32_t *islong) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < S; k += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t b = sptr[k], len = sptr[k + 1] - b;
     const bool lng = len > chunk;
     bool head = (k == 0) || lng;
     if (k > 0) {
       const uint32_t pb = sptr[k - 1], plen = b - pb;
-      head = head || plen > chunk || (b / chunk) != (pb / chunk);
+      head = head || plen > chunk || (b / run) != (pb / run);
     }
     nu[k] = lng ? (len + chunk - 1) / chunk : (head ? 1u : 0u);
     islong[k] = lng ? 1u : 0u;
   }
 }
 
-__global__ void unit_write_kernel(int64_t S, const uint32_t *sptr, uint32_t chunk, const uint32_t *nu,
+__global__ void unit_write_kernel(int64_t S, const uint32_t *sptr, const uint32_t *nu,
                                   const uint32_t *uoff, const uint32_t *islong, const uint32_t *lid,
                                   uint32_t *unit_e0, uint32_t *unit_k0, int32_t *unit_slot, uint32_t *long_k,
                                   uint32_t *long_u0, uint32_t *long_np) {
@@ -635,21 +636,35 @@ __global__ void unit_long_kernel(int64_t n_long, const uint32_t *long_k, const u
   }
 }
 
-// Nonzeros per work unit: about 64 units for each SM (four to six rounds of the warps it
-// holds, so that the last one is short), at most 2,048 nonzeros (fewer slices cut), at least
-// 128 (a slice of 100 stays whole).  Eight units per SM and at least 256 left SMs idle: 5M
-// nonzeros, ranks 8^4, four modes 1.24 -> 1.04 ms; 600,011 nonzeros, ranks 12 x 7 x 20 at 2,048,
-// 1,024, 512, 256, 128 nonzeros: 0.51, 0.31, 0.18, 0.13, 0.12 ms.
-static int pick_chunk(int64_t nnz, int num_sms) {
+// Nonzeros per work unit of a mode: slices longer than `chunk` are cut into pieces of it, and
+// shorter ones are run together while they start in the same multiple of `run`.
+//   run     about 64 units for each SM (several rounds of the warps it holds, so that the last
+//           one is short), 32 to 2,048 nonzeros.  Eight units per SM and at least 256 nonzeros
+//           left SMs idle: 5M nonzeros, ranks 8^4, four modes 1.24 -> 1.04 ms; 600,011 nonzeros,
+//           ranks 12 x 7 x 20, at 2,048, 1,024, 512, 256, 128 nonzeros: 0.51, 0.31, 0.18, 0.13,
+//           0.12 ms; below 128 only slices that are as short share a unit (each costs its warp
+//           the latency of finishing a row).
+//   chunk   at least 128 (256 where that still makes eight units per SM: half the partial rows;
+//           589,320 nonzeros in 43 to 1,678 slices, BF16, three modes 61 us, at 128 65 us), and
+//           1.5 times the mode's average slice up to 256: slices of about the same length stay
+//           whole, which saves the kernel that adds the pieces (10,000 nonzeros, slices of 100:
+//           11 us a mode, cut at 64 13 us).
+struct UnitSize {
+  int chunk, run;
+};
+static UnitSize pick_units(int64_t nnz, int64_t slices, int num_sms) {
   const char *f = std::getenv("TUCKER_TTMC_CHUNK");
   if (f) {
     int v = std::atoi(f);
-    if (v >= 32 && v <= (1 << 20) && (v % 32) == 0) return v;
+    if (v >= 32 && v <= (1 << 20) && (v % 32) == 0) return {v, v};
   }
-  int64_t target = nnz / ((int64_t)num_sms * 64);
-  int chunk = 128;
-  while (chunk < 2048 && (int64_t)chunk * 2 <= target) chunk *= 2;
-  return chunk;
+  const int64_t target = nnz / ((int64_t)num_sms * 64);
+  UnitSize u{0, 32};
+  while (u.run < 2048 && (int64_t)u.run * 2 <= target) u.run *= 2;
+  u.chunk = std::max(nnz >= (int64_t)num_sms * 8 * 256 ? 256 : 128, u.run);
+  const int64_t whole = (3 * nnz / (2 * std::max<int64_t>(slices, 1)) + 31) / 32 * 32;
+  if (whole <= 256) u.chunk = std::max(u.chunk, (int)whole);
+  return u;
 }
 
 // RAII holder for temporaries of the build
@@ -697,12 +712,13 @@ struct UnitTables {
   int64_t *n_units, *n_long;
 };
 
-static tucker_status build_units(Ctx *c, int64_t S, const uint32_t *ptr, int chunk, uint32_t *nu, uint32_t *islong,
+static tucker_status build_units(Ctx *c, int64_t S, const uint32_t *ptr, UnitSize size, uint32_t *nu, uint32_t *islong,
                                  uint32_t *uoff, uint32_t *lid, uint32_t *stmp, uint32_t *d_small, UnitTables o,
                                  cudaStream_t s) {
+  const uint32_t chunk = (uint32_t)size.chunk, run = (uint32_t)size.run;
   uint32_t nunits = 0, nlong = 0;
   if (S > 0) {
-    unit_count_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, (uint32_t)chunk, nu, islong);
+    unit_count_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, chunk, run, nu, islong);
     ::tk::count_launch();
     exclusive_scan_total(nu, uoff, S, stmp, d_small + 2, s);
     exclusive_scan_total(islong, lid, S, stmp, d_small + 3, s);
@@ -721,12 +737,12 @@ static tucker_status build_units(Ctx *c, int64_t S, const uint32_t *ptr, int chu
   TK_TRY(dev_alloc(c, o.long_u0, (size_t)std::max<uint32_t>(nlong, 1)));
   TK_TRY(dev_alloc(c, o.long_np, (size_t)std::max<uint32_t>(nlong, 1)));
   if (S > 0) {
-    unit_write_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, (uint32_t)chunk, nu, uoff, islong, lid, *o.e0, *o.k0,
+    unit_write_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, nu, uoff, islong, lid, *o.e0, *o.k0,
                                                    *o.slot, *o.long_k, *o.long_u0, *o.long_np);
     ::tk::count_launch();
     if (nlong > 0) {
       unit_long_kernel<<<(unsigned)std::min<uint32_t>(nlong, (uint32_t)c->num_sms * 4), 256, 0, s>>>(
-          nlong, *o.long_k, *o.long_u0, *o.long_np, ptr, (uint32_t)chunk, *o.e0, *o.k0, *o.slot);
+          nlong, *o.long_k, *o.long_u0, *o.long_np, ptr, chunk, *o.e0, *o.k0, *o.slot);
       ::tk::count_launch();
     }
   }
@@ -924,7 +940,6 @@ tucker_status build_sorted_copies(Ctx *c, const uint32_t *coords_in, const float
         mc.other[t++] = m;
         mc.P *= c->ranks[m];
       }
-    mc.chunk = pick_chunk(Z, c->num_sms);
     if (n == 0) {  // the lexicographic order is already sorted by i_1: mode 1 reads the
                    // coalesced arrays themselves (read-only after the initialisation)
       rows[0] = c->coords;
@@ -1000,7 +1015,9 @@ tucker_status build_sorted_copies(Ctx *c, const uint32_t *coords_in, const float
     {
       UnitTables o{&mc.unit_e0, &mc.unit_k0, &mc.long_k, &mc.long_u0, &mc.long_np, &mc.unit_slot, &mc.n_units,
                    &mc.n_long};
-      tucker_status st2 = build_units(c, S, mc.sptr, mc.chunk, nu, islong, uoff, lid, stmp, d_small, o, s);
+      const UnitSize size = pick_units(Z, S, c->num_sms);
+      mc.chunk = size.chunk;
+      tucker_status st2 = build_units(c, S, mc.sptr, size, nu, islong, uoff, lid, stmp, d_small, o, s);
       if (st2 != TUCKER_OK) return st2;
     }
   }
@@ -1133,7 +1150,7 @@ tucker_status build_sorted_copies(Ctx *c, const uint32_t *coords_in, const float
       }
       UnitTables o{&mc.funit_e0, &mc.funit_k0, &mc.flong_k, &mc.flong_u0, &mc.flong_np, &mc.funit_slot,
                    &mc.fn_units, &mc.fn_long};
-      st2 = build_units(c, mc.S, mc.fsptr, mc.fchunk, nu, islong, uoff, lid, stmp, d_small, o, s);
+      st2 = build_units(c, mc.S, mc.fsptr, {mc.fchunk, mc.fchunk}, nu, islong, uoff, lid, stmp, d_small, o, s);
       if (st2 != TUCKER_OK) return st2;
     } else {  // the nonzero form does not depend on the order within a slice
       mc.fmid_t = 0;
