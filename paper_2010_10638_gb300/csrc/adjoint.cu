@@ -6,10 +6,13 @@
 //     dL/dG_(1) = U_1^T TTMc_1(E)          (the core-tensor contraction of Section III-B)
 // and the forward pass needs only one row of Q = U_1 G_(1) per slice:
 //     xhat_z = < Q(i_1(z), :), kron_{m > 1} U_m(i_m(z), :) >.
-// So the adjoint is: one small dense product (Q), one pass over the nonzeros for the
-// residuals and the loss, then for every mode a TTMc of the residuals (the kernel of
-// ttmc.cu, fed with the caller's FP32 factors) and two small dense contractions.
-// Kronecker rows are recomputed, never stored; every reduction has a fixed order.
+// So the adjoint is: one small dense product (Q), one pass over mode 1's nonzeros for the
+// residuals, the loss and the TTMc of the residuals (ttmc_tile.cuh: the gathers are what it
+// costs, so they are made once), then for every other mode a TTMc of the residuals (the
+// kernels of ttmc.cu, fed with the caller's FP32 factors; the tiled one reads the residuals
+// in place through the source positions, 10M observations 1.34 ms a step against 1.44 ms with
+// a gather before it) and small dense contractions.  Kronecker rows are recomputed, never
+// stored; every reduction has a fixed order.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -92,19 +95,6 @@ __global__ void __launch_bounds__(256) adj_forward_kernel(AdjFwd a) {
   if (threadIdx.x == 0) a.part[blockIdx.x] = red[0];
 }
 
-__global__ void adj_loss_kernel(const double *part, int np, double *loss) {
-  __shared__ double red[256];
-  double t = 0.0;
-  for (int i = threadIdx.x; i < np; i += blockDim.x) t += part[i];
-  red[threadIdx.x] = t;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *loss = 0.5 * red[0];
-}
-
 __global__ void adj_gather_kernel(int64_t Z, const uint32_t *src, const float *e0, float *en) {
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < Z; p += (int64_t)gridDim.x * blockDim.x)
     en[p] = e0[src[p]];
@@ -134,8 +124,8 @@ __global__ void adj_unfold_kernel(Unfold u, const float *G, int64_t PR, float *G
   }
 }
 
-// dU[i, r] = sum_c Y[i, c] Gn[r, c]
-__global__ void adj_du_kernel(const float *Y, const float *Gn, int64_t I, int64_t P, int R, float *dU) {
+// dU[i, r] = sum_c Y[i, c] Gn[r, c], one thread per entry; for P and R too large for adj_du_kernel
+__global__ void adj_du_wide_kernel(const float *Y, const float *Gn, int64_t I, int64_t P, int R, float *dU) {
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < I * R;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = idx / R;
@@ -148,29 +138,152 @@ __global__ void adj_du_kernel(const float *Y, const float *Gn, int64_t I, int64_
   }
 }
 
-// split-K partials of dG[r, c] = sum_i U1[i, r] Y[i, c]  (outputs r*P + c)
-__global__ void adj_dg_partial_kernel(const float *U1, const float *Y, int64_t I, int R, int64_t P, int rows_per,
-                                      float *gpart) {
-  const int64_t out = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (out >= (int64_t)R * P) return;
-  const int r = (int)(out / P);
-  const int64_t c = out % P;
-  const int64_t i0 = (int64_t)blockIdx.y * rows_per, i1 = std::min<int64_t>(I, i0 + rows_per);
-  float t = 0.f;
-  for (int64_t i = i0; i < i1; ++i) t = fmaf(U1[i * R + r], Y[i * P + c], t);
-  gpart[(int64_t)blockIdx.y * R * P + out] = t;
+// The same with G_(n) (transposed, read from G in place) and a tile of rows of Y in shared
+// memory: threads (row, r) with r fastest, so a warp reads one or a few rows of Y (four
+// columns at a time, the same address for all r) and adjacent entries of G.  Y is read once,
+// coalesced, and G_(n) needs no kernel and no copy of its own.
+constexpr int kDuThreads = 256;
+__host__ __device__ inline int du_stride(int P) { return (P + 3) / 4 * 4 + 4; }  // rows in different banks
+__global__ void __launch_bounds__(kDuThreads) adj_du_kernel(const float *__restrict__ Y, const float *__restrict__ G,
+                                                            Unfold u, int64_t I, int P, int nr,
+                                                            float *__restrict__ dU) {
+  extern __shared__ float4 du_smem[];
+  const int R = u.R[u.n], ld = du_stride(P);
+  float *ys = reinterpret_cast<float *>(du_smem);  // [nr][ld]
+  float *gs = ys + nr * ld;                        // [P][R]
+  for (int q = threadIdx.x; q < P * R; q += kDuThreads) {
+    int c = q / R, off = 0, stride = 1;
+    for (int m = u.N - 1; m >= 0; --m) {  // C-order place of (c, r) in G
+      const int i = m == u.n ? q % R : c % u.R[m];
+      if (m != u.n) c /= u.R[m];
+      off += i * stride;
+      stride *= u.R[m];
+    }
+    gs[q] = __ldg(G + off);
+  }
+  const int row = (int)threadIdx.x / R, r = (int)threadIdx.x % R;
+  for (int64_t i0 = (int64_t)blockIdx.x * nr; i0 < I; i0 += (int64_t)gridDim.x * nr) {
+    const int rows = (int)min((int64_t)nr, I - i0);
+    if (i0 != (int64_t)blockIdx.x * nr) __syncthreads();  // the previous tile is read
+#pragma unroll 4
+    for (int q = threadIdx.x; q < rows * P; q += kDuThreads) ys[q / P * ld + q % P] = __ldg(Y + i0 * P + q);
+    __syncthreads();  // (the first time, G is there too)
+    if (row < rows) {
+      const float *y = ys + row * ld, *g = gs + r;
+      float t = 0.f;
+      int c = 0;
+      for (; c + 3 < P; c += 4) {
+        const float4 q = *reinterpret_cast<const float4 *>(y + c);
+        t = fmaf(q.x, g[c * R], t);
+        t = fmaf(q.y, g[(c + 1) * R], t);
+        t = fmaf(q.z, g[(c + 2) * R], t);
+        t = fmaf(q.w, g[(c + 3) * R], t);
+      }
+      for (; c < P; ++c) t = fmaf(y[c], g[c * R], t);
+      dU[(i0 + row) * R + r] = t;
+    }
+  }
 }
 
-__global__ void adj_dg_reduce_kernel(const float *gpart, int chunks, int64_t RP, float *dG) {
-  for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < RP; o += (int64_t)gridDim.x * blockDim.x) {
+// Row-range partials of dG[r, c] = sum_i U1[i, r] Y[i, c]: a thread owns column c and eight
+// ranks for every fourth row of its range, so Y is read once per eight ranks and U's entries
+// are the same for a whole warp; the four row lanes are added in order.  At most 256 ranges of
+// at least 16 rows: bound by the latency of a thread's chain of loads, so the chains are kept
+// short (ncu, cold caches: 20,000 rows, 100 columns, 10 ranks, 20 rows a thread, 19 us, as 313 a
+// thread 75 us; 200 rows, 64 columns, 8 ranks 5 us, as one chain of 200 48 us).
+constexpr int kDgRanks = 8, kDgCols = 64, kDgLanes = 4, kDgChunks = 256;
+__global__ void __launch_bounds__(kDgCols *kDgLanes) adj_dg_partial_kernel(const float *__restrict__ U1,
+                                                                           const float *__restrict__ Y, int64_t I,
+                                                                           int R, int64_t P, int rows_per,
+                                                                           float *__restrict__ gpart) {
+  __shared__ float part[kDgLanes - 1][kDgRanks][kDgCols];
+  const int cl = (int)threadIdx.x % kDgCols, rl = (int)threadIdx.x / kDgCols;
+  const int64_t c = (int64_t)blockIdx.x * kDgCols + cl;
+  const int r0 = (int)blockIdx.z * kDgRanks, nr = min(kDgRanks, R - r0);
+  const int64_t i0 = (int64_t)blockIdx.y * rows_per, i1 = min(I, i0 + rows_per);
+  float t[kDgRanks];
+#pragma unroll
+  for (int k = 0; k < kDgRanks; ++k) t[k] = 0.f;
+  if (c < P) {
+#pragma unroll 4
+    for (int64_t i = i0 + rl; i < i1; i += kDgLanes) {
+      const float y = __ldg(Y + i * P + c);
+#pragma unroll
+      for (int k = 0; k < kDgRanks; ++k) t[k] = fmaf(k < nr ? __ldg(U1 + i * R + r0 + k) : 0.f, y, t[k]);
+    }
+  }
+  if (rl > 0) {
+#pragma unroll
+    for (int k = 0; k < kDgRanks; ++k) part[rl - 1][k][cl] = t[k];
+  }
+  __syncthreads();
+  if (rl > 0 || c >= P) return;
+#pragma unroll
+  for (int k = 0; k < kDgRanks; ++k) {
+    if (k >= nr) break;
+    for (int l = 0; l < kDgLanes - 1; ++l) t[k] += part[l][k][cl];
+    gpart[((int64_t)blockIdx.y * R + r0 + k) * P + c] = t[k];
+  }
+}
+
+// dG from its partials, a warp per entry (lanes take every 32nd range, then a tree); the last
+// block adds the loss from its partials.
+__global__ void __launch_bounds__(256) adj_finish_kernel(const float *__restrict__ gpart, int chunks, int64_t RP,
+                                                         float *__restrict__ dG, const double *__restrict__ part,
+                                                         int64_t np, double *__restrict__ loss) {
+  if (blockIdx.x == gridDim.x - 1) {
+    __shared__ double red[256];
+    double t = 0.0;
+    for (int64_t i = threadIdx.x; i < np; i += 256) t += part[i];
+    red[threadIdx.x] = t;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+      if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = 0.5 * red[0];
+    return;
+  }
+  const int lane = threadIdx.x & 31;
+  for (int64_t o = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); o < RP; o += (int64_t)(gridDim.x - 1) * 8) {
     float t = 0.f;
-    for (int q = 0; q < chunks; ++q) t += gpart[(int64_t)q * RP + o];
-    dG[o] = t;
+    for (int q = lane; q < chunks; q += 32) t += __ldg(gpart + (int64_t)q * RP + o);
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) t += __shfl_xor_sync(0xffffffffu, t, h);
+    if (lane == 0) dG[o] = t;
   }
 }
 
 static unsigned blocks_for(int64_t n, int64_t cap = 65535LL * 8) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, cap));
+}
+
+// dU_n from Y_(n) of the residuals
+static cudaError_t launch_du(Ctx *c, int n, const float *G, int64_t PR, float *dU, cudaStream_t s) {
+  const ModeCopy &mc = c->mode[n];
+  const int R = c->ranks[n];
+  Unfold uf{};
+  uf.N = c->N;
+  uf.n = n;
+  for (int m = 0; m < c->N; ++m) uf.R[m] = c->ranks[m];
+  const int nr = kDuThreads / R;
+  const int64_t smem = ((int64_t)nr * (mc.P + 8) + mc.P * R) * (int64_t)sizeof(float);
+  if (smem <= 200 * 1024) {
+    const size_t bytes = (size_t)(nr * du_stride((int)mc.P) + (int)mc.P * R) * sizeof(float);
+    const cudaError_t e = cudaFuncSetAttribute(adj_du_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return e;
+    const int64_t tiles = (mc.I + nr - 1) / nr;
+    const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(4, (int64_t)(220 * 1024) / (int64_t)bytes));
+    const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, c->num_sms * per_sm));
+    adj_du_kernel<<<blocks, kDuThreads, bytes, s>>>(c->adj_Y, G, uf, mc.I, (int)mc.P, nr, dU);
+    ::tk::count_launch();
+  } else {
+    adj_unfold_kernel<<<blocks_for(PR), 256, 0, s>>>(uf, G, PR, c->adj_Gn);
+    ::tk::count_launch();
+    adj_du_wide_kernel<<<blocks_for(mc.I * R), 256, 0, s>>>(c->adj_Y, c->adj_Gn, mc.I, mc.P, R, dU);
+    ::tk::count_launch();
+  }
+  return cudaGetLastError();
 }
 
 tucker_status launch_loss_grad(Ctx *c, const float *const *U, const float *G, double *loss, float *const *dU,
@@ -180,21 +293,25 @@ tucker_status launch_loss_grad(Ctx *c, const float *const *U, const float *G, do
   int64_t PR = 1, ymax = 1;
   for (int m = 0; m < N; ++m) PR *= c->ranks[m];
   for (int m = 0; m < N; ++m) ymax = std::max(ymax, c->mode[m].I * c->mode[m].P);
-  const int64_t I1 = c->dims[0], P1 = c->mode[0].P;
+  const ModeCopy &m0 = c->mode[0];
+  const int64_t I1 = c->dims[0], P1 = m0.P;
   const int R1 = c->ranks[0];
-  const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>(64, (I1 + 255) / 256));
+  const int64_t room = std::max<int64_t>(1, (64ll << 20) / PR);  // partials of dG: 256 MB at most
+  const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>({kDgChunks, (I1 + 15) / 16, room}));
+  int64_t qrow = 0;  // floats of a row of Q for the fused form
+  const bool fused = tile_adj_plan(tile_call(c, 0, nullptr, nullptr), &qrow) && m0.n_units > 0;
   if (!c->adj_e0) {  // first call: buffers allocated in the order of s, ready for any stream after the sync
     c->astream = s;
-    TK_CUDA(dev_alloc(c, &c->adj_e0, (size_t)std::max<int64_t>(Z, 1)));
     TK_CUDA(dev_alloc(c, &c->adj_en, (size_t)std::max<int64_t>(Z, 1)));
     TK_CUDA(dev_alloc(c, &c->adj_Y, (size_t)ymax));
-    TK_CUDA(dev_alloc(c, &c->adj_Q, (size_t)(I1 * P1)));
+    TK_CUDA(dev_alloc(c, &c->adj_Q, (size_t)(I1 * (fused ? qrow : P1))));
     TK_CUDA(dev_alloc(c, &c->adj_Gn, (size_t)PR));
     int64_t packed = 0;
     for (int m = 0; m < N; ++m) packed += c->dims[m] * tile_layout(c->ranks[m]).row();
     TK_CUDA(dev_alloc(c, &c->adj_U, (size_t)packed));
-    TK_CUDA(dev_alloc(c, &c->adj_part, (size_t)kAdjRedBlocks));
-    TK_CUDA(dev_alloc(c, &c->adj_gpart, (size_t)(64 * PR)));
+    TK_CUDA(dev_alloc(c, &c->adj_part, (size_t)std::max<int64_t>(kAdjRedBlocks, m0.n_units)));
+    TK_CUDA(dev_alloc(c, &c->adj_gpart, (size_t)(chunks * PR)));
+    TK_CUDA(dev_alloc(c, &c->adj_e0, (size_t)std::max<int64_t>(Z, 1)));
     TK_CUDA(cudaStreamSynchronize(s));
     c->astream = 0;
   }
@@ -218,52 +335,66 @@ tucker_status launch_loss_grad(Ctx *c, const float *const *U, const float *G, do
     }
     if (copies) launch_tile_pack(pk, copies, s);
   }
-  // (1) Q = U_1 G_(1)
-  adj_q_kernel<<<blocks_for(I1 * P1), 256, 0, s>>>(U[0], G, I1, R1, P1, c->adj_Q);
-  ::tk::count_launch();
-  // (2) residuals and the loss
-  AdjFwd f{};
-  f.N = N;
-  f.Z = Z;
-  f.coords = c->coords;
-  f.vals = c->vals;
-  for (int m = 0; m < N; ++m) {
-    f.U[m] = U[m];
-    f.R[m] = c->ranks[m];
+  // (1) residuals, their squares, and for mode 1 the TTMc of the residuals: in one kernel, or
+  //     where a row has more tiles than that holds, Q = U_1 G_(1), then one thread per nonzero
+  int64_t parts = kAdjRedBlocks;
+  if (fused) {
+    TileAdj a{};
+    a.U = U[0];
+    a.G = G;
+    a.I = I1;
+    a.R = R1;
+    a.Q = c->adj_Q;
+    a.esrc = m0.src;
+    a.e_out = c->adj_e0;
+    a.sq_part = c->adj_part;
+    TK_CUDA(launch_tile_adj(tile_call(c, 0, Up, c->adj_Y), a, s));
+    ttmc_finish(c, 0, c->adj_Y, nullptr, s);
+    TK_CUDA(cudaGetLastError());
+    parts = m0.n_units;
+  } else {
+    adj_q_kernel<<<blocks_for(I1 * P1), 256, 0, s>>>(U[0], G, I1, R1, P1, c->adj_Q);
+    ::tk::count_launch();
+    AdjFwd f{};
+    f.N = N;
+    f.Z = Z;
+    f.coords = c->coords;
+    f.vals = c->vals;
+    for (int m = 0; m < N; ++m) {
+      f.U[m] = U[m];
+      f.R[m] = c->ranks[m];
+    }
+    f.Q = c->adj_Q;
+    f.P = P1;
+    f.e = c->adj_e0;
+    f.part = c->adj_part;
+    adj_forward_kernel<<<kAdjRedBlocks, 256, 0, s>>>(f);
+    ::tk::count_launch();
   }
-  f.Q = c->adj_Q;
-  f.P = P1;
-  f.e = c->adj_e0;
-  f.part = c->adj_part;
-  adj_forward_kernel<<<kAdjRedBlocks, 256, 0, s>>>(f);
-  ::tk::count_launch();
-  adj_loss_kernel<<<1, 256, 0, s>>>(c->adj_part, kAdjRedBlocks, loss);
-  ::tk::count_launch();
-  // (3) per mode: TTMc of the residuals, then dU_n and (mode 1) dG
+  // (2) per mode: TTMc of the residuals, then dU_n and (mode 1) dG and the loss
   for (int n = 0; n < N; ++n) {
     const ModeCopy &mc = c->mode[n];
-    const float *en = c->adj_e0;
-    if (mc.src && Z > 0) {  // this mode's order is not the lexicographic one
-      adj_gather_kernel<<<blocks_for(Z, 4096), 256, 0, s>>>(Z, mc.src, c->adj_e0, c->adj_en);
-      ::tk::count_launch();
-      en = c->adj_en;
+    if (!(n == 0 && fused)) {
+      const float *en = c->adj_e0;
+      const uint32_t *src = mc.src;  // where this mode's order is not the lexicographic one
+      if (src && Z > 0 && !ttmc_tiled(c, n)) {
+        adj_gather_kernel<<<blocks_for(Z, 4096), 256, 0, s>>>(Z, src, c->adj_e0, c->adj_en);
+        ::tk::count_launch();
+        en = c->adj_en;
+        src = nullptr;
+      }
+      tucker_status st = launch_ttmc_ex(c, n, c->adj_Y, en, src, Up, s);
+      if (st != TUCKER_OK) return st;
     }
-    tucker_status st = launch_ttmc_ex(c, n, c->adj_Y, en, Up, s);
-    if (st != TUCKER_OK) return st;
-    Unfold uf{};
-    uf.N = N;
-    uf.n = n;
-    for (int m = 0; m < N; ++m) uf.R[m] = c->ranks[m];
-    adj_unfold_kernel<<<blocks_for(PR), 256, 0, s>>>(uf, G, PR, c->adj_Gn);
-    ::tk::count_launch();
-    adj_du_kernel<<<blocks_for(mc.I * c->ranks[n]), 256, 0, s>>>(c->adj_Y, c->adj_Gn, mc.I, mc.P, c->ranks[n], dU[n]);
-    ::tk::count_launch();
+    TK_CUDA(launch_du(c, n, G, PR, dU[n], s));
     if (n == 0) {
       const int rows_per = (int)((I1 + chunks - 1) / chunks);
-      adj_dg_partial_kernel<<<dim3((unsigned)((R1 * P1 + 255) / 256), (unsigned)chunks), 256, 0, s>>>(
-          U[0], c->adj_Y, I1, R1, P1, rows_per, c->adj_gpart);
+      const dim3 grid((unsigned)((P1 + kDgCols - 1) / kDgCols), (unsigned)chunks,
+                      (unsigned)((R1 + kDgRanks - 1) / kDgRanks));
+      adj_dg_partial_kernel<<<grid, kDgCols * kDgLanes, 0, s>>>(U[0], c->adj_Y, I1, R1, P1, rows_per, c->adj_gpart);
       ::tk::count_launch();
-      adj_dg_reduce_kernel<<<blocks_for(PR), 256, 0, s>>>(c->adj_gpart, chunks, PR, dG);
+      adj_finish_kernel<<<(unsigned)std::min<int64_t>((PR + 7) / 8, 2048) + 1, 256, 0, s>>>(
+          c->adj_gpart, chunks, PR, dG, c->adj_part, parts, loss);
       ::tk::count_launch();
     }
   }

@@ -137,11 +137,11 @@ struct Ctx {
   float *adj_e0 = nullptr;     // residuals in lexicographic order
   float *adj_en = nullptr;     // residuals in the order of one mode's copy
   float *adj_Y = nullptr;      // TTMc of the residual tensor (max I_n * P_n)
-  float *adj_Q = nullptr;      // U_1 G_(1) (I_1 x P_1)
+  float *adj_Q = nullptr;      // U_1 G_(1) (I_1 x P_1, or in the order of the tiled form's lanes)
   float *adj_Gn = nullptr;     // one unfolding of G (prod R)
   float *adj_U = nullptr;      // the caller's factors in tile_layout, one after another
   double *adj_part = nullptr;  // loss partials
-  float *adj_gpart = nullptr;  // split-K partials of dL/dG
+  float *adj_gpart = nullptr;  // row-range partials of dL/dG
   bool G_valid = false;
   int sweeps = 0;
 
@@ -223,9 +223,13 @@ int32_t qrp_check_site();                 // checked build: first index check th
 void make_factor_maps(Ctx *c);
 // 0, 1, ..., n-1 and n ones (the index and value streams of the fiber form's update pass)
 void fill_iota_ones(uint32_t *iota, float *ones, int64_t n, cudaStream_t s);
-// TTMc of mode `mode` with values `val` (in that mode's sorted order) and FP32 factors
-// Uf[m] (indexed by mode; Uf[mode] unused) instead of the context's own.
-tucker_status launch_ttmc_ex(Ctx *c, int mode, float *Y, const float *val, const float *const *Uf, cudaStream_t s);
+// TTMc of mode `mode` with the value of sorted position e val[e] (or val[vsrc[e]], only where
+// ttmc_tiled) and FP32 factors Uf[m] (indexed by mode, in tile_layout and 16-byte aligned;
+// Uf[mode] unused) instead of the context's own.
+tucker_status launch_ttmc_ex(Ctx *c, int mode, float *Y, const float *val, const uint32_t *vsrc,
+                             const float *const *Uf, cudaStream_t s);
+bool ttmc_tiled(const Ctx *c, int mode);  // the FP32 TTMc of this mode runs the tiled form
+void ttmc_finish(Ctx *c, int mode, float *Y, float2 *sq, cudaStream_t s);  // cut slices' rows, empty rows
 
 // ---- K-b, tiled form (ttmc_tile.cuh): FP32, any order and ranks
 // A factor copy for it: the R ranks in n = 1, 2, 4 or 8 chunks of at most T <= 8, of which
@@ -275,6 +279,20 @@ struct TileCall {
   int num_sms;
 };
 cudaError_t launch_ttmc_tile(const TileCall &c, cudaStream_t s);
+TileCall tile_call(const Ctx *c, int mode, const float *const *Uf, float *Y);  // (the tensor's values)
+// adjoint form: the TTMc of e_z = <(U G_(n))(i_n, :), kron rows of z> - val_z, with the e_z
+// written out and their squares summed per work unit (c.val: the tensor's values)
+struct TileAdj {
+  const float *U, *G;    // this mode's factor (I x R, plain) and the core as G_(n) (R x P)
+  int64_t I;
+  int R;
+  float *Q;              // workspace: I rows of tile_adj_plan's floats
+  const uint32_t *esrc;  // e of sorted position p goes to e_out[esrc[p]], or e_out[p] with esrc null
+  float *e_out;
+  double *sq_part;       // [c.n_units]
+};
+bool tile_adj_plan(const TileCall &c, int64_t *row_floats);  // false: not covered
+cudaError_t launch_tile_adj(const TileCall &c, const TileAdj &a, cudaStream_t s);
 struct TilePack {  // plain row-major factors to copies in tile_layout
   const float *in[kMaxOrder];
   float *out[kMaxOrder];

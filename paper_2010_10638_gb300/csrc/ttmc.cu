@@ -1631,10 +1631,54 @@ static bool fused_fibers() {
   return e && e[0] == '1';
 }
 
+TileCall tile_call(const Ctx *c, int mode, const float *const *Uf, float *Y) {
+  const ModeCopy &mc = c->mode[mode];
+  TileCall t{};
+  t.nother = mc.nother;
+  for (int q = 0; q < mc.nother; ++q) {
+    const int m = mc.other[q];
+    t.idx[q] = mc.idx[q];
+    t.U[q] = Uf ? Uf[m] : c->U32[m];
+    t.R[q] = c->ranks[m];
+  }
+  t.val = mc.val;
+  t.sptr = mc.sptr;
+  t.sid = mc.sid;
+  t.S = (uint32_t)mc.S;
+  t.unit_e0 = mc.unit_e0;
+  t.unit_k0 = mc.unit_k0;
+  t.unit_slot = mc.unit_slot;
+  t.n_units = mc.n_units;
+  t.Z = (uint32_t)c->nnz;
+  t.Y = Y;
+  t.carry = c->carry;
+  t.P = mc.P;
+  t.slice_len = (double)c->nnz / (double)std::max<int64_t>(mc.S, 1);
+  t.num_sms = c->num_sms;
+  return t;
+}
+
+bool ttmc_tiled(const Ctx *c, int mode) {
+  const ModeCopy &mc = c->mode[mode];
+  return !(mc.nother == 2 && pipe_shape(c->ranks[mc.other[0]], c->ranks[mc.other[1]]));
+}
+
+// What the nonzero forms leave to do: rows of slices cut over several units, empty rows.
+void ttmc_finish(Ctx *c, int mode, float *Y, float2 *sq, cudaStream_t s) {
+  const ModeCopy &mc = c->mode[mode];
+  if (mc.n_long > 0) launch_fixup(mc.long_k, mc.long_u0, mc.long_np, mc.n_long, mc.sid, c->carry, Y, mc.P, s, sq);
+  if (mc.n_empty > 0) {
+    ttmc_zero_rows_kernel<<<(unsigned)std::min<int64_t>(mc.n_empty, 65535), 256, 0, s>>>(mc.empty, mc.n_empty, Y,
+                                                                                        mc.P);
+    ::tk::count_launch();
+  }
+}
+
 // With `colsq` given, the pipelined FP32 forms also write the column sums of squares of Y
 // there (*norms true); every other form leaves *norms false.
-static tucker_status ttmc_impl(Ctx *c, int mode, float *Y, const float *val, const float *const *Uf,
-                               cudaStream_t s, double *colsq = nullptr, bool *norms = nullptr) {
+static tucker_status ttmc_impl(Ctx *c, int mode, float *Y, const float *val, const uint32_t *vsrc,
+                               const float *const *Uf, cudaStream_t s, double *colsq = nullptr,
+                               bool *norms = nullptr) {
   const ModeCopy &mc = c->mode[mode];
   if (norms) *norms = false;
   // per-block pairs of P columns for each of the 8 warps: formed where that stays small
@@ -1692,12 +1736,7 @@ static tucker_status ttmc_impl(Ctx *c, int mode, float *Y, const float *val, con
                            : dispatch_fiber<float>(f, p.R[ft], p.R[1 - ft], ft == 0, s, &err);
     if (done) {
       TK_CUDA(err);
-      if (mc.n_long > 0) launch_fixup(mc.long_k, mc.long_u0, mc.long_np, mc.n_long, mc.sid, c->carry, Y, mc.P, s);
-      if (mc.n_empty > 0) {
-        ttmc_zero_rows_kernel<<<(unsigned)std::min<int64_t>(mc.n_empty, 65535), 256, 0, s>>>(mc.empty, mc.n_empty,
-                                                                                            Y, mc.P);
-        ::tk::count_launch();
-      }
+      ttmc_finish(c, mode, Y, nullptr, s);
       TK_CUDA(cudaGetLastError());
       return TUCKER_OK;
     }
@@ -1781,46 +1820,19 @@ static tucker_status ttmc_impl(Ctx *c, int mode, float *Y, const float *val, con
     // 5M nonzeros, ranks 8^4 1.03 ms (4 x 4 tiles, Kronecker rows staged: 2.08 ms); 10M
     // nonzeros, ranks 10^3 0.90 ms (9.9 ms).
     if (!done) {
-      TileCall t{};
-      t.nother = mc.nother;
-      for (int q = 0; q < mc.nother; ++q) {
-        const int m = mc.other[q];
-        t.idx[q] = mc.idx[q];
-        t.U[q] = Uf ? Uf[m] : c->U32[m];
-        t.R[q] = c->ranks[m];
-      }
+      TileCall t = tile_call(c, mode, Uf, Y);
       t.val = p.val;
-      t.sptr = mc.sptr;
-      t.sid = mc.sid;
-      t.S = (uint32_t)mc.S;
-      t.unit_e0 = mc.unit_e0;
-      t.unit_k0 = mc.unit_k0;
-      t.unit_slot = mc.unit_slot;
-      t.n_units = mc.n_units;
-      t.Z = p.Z;
-      t.Y = Y;
-      t.carry = c->carry;
-      t.P = mc.P;
-      t.slice_len = (double)c->nnz / (double)std::max<int64_t>(mc.S, 1);
-      t.num_sms = c->num_sms;
+      t.vsrc = vsrc;
       err = launch_ttmc_tile(t, s);
     }
     TK_CUDA(err);
   }
-  if (mc.n_long > 0) {
-    launch_fixup(mc.long_k, mc.long_u0, mc.long_np, mc.n_long, mc.sid, c->carry, Y, mc.P, s, sq_fix);
-    TK_CUDA(cudaGetLastError());
-  }
+  ttmc_finish(c, mode, Y, sq_fix, s);
+  TK_CUDA(cudaGetLastError());
   if (sq_rows > 0) {
     launch_colsq(c->sq_part, sq_rows, mc.P, c->sq_cnt, colsq, s);
     TK_CUDA(cudaGetLastError());
     *norms = true;
-  }
-  if (mc.n_empty > 0) {
-    ttmc_zero_rows_kernel<<<(unsigned)std::min<int64_t>(mc.n_empty, 65535), 256, 0, s>>>(mc.empty, mc.n_empty, Y,
-                                                                                        mc.P);
-    ::tk::count_launch();
-    TK_CUDA(cudaGetLastError());
   }
   return TUCKER_OK;
 }
@@ -1856,15 +1868,16 @@ void make_factor_maps(Ctx *c) {
 }
 
 tucker_status launch_ttmc(Ctx *c, int mode, float *Y, cudaStream_t s) {
-  return ttmc_impl(c, mode, Y, nullptr, nullptr, s);
+  return ttmc_impl(c, mode, Y, nullptr, nullptr, nullptr, s);
 }
 
 tucker_status launch_ttmc_norms(Ctx *c, int mode, float *Y, double *colsq, bool *formed, cudaStream_t s) {
-  return ttmc_impl(c, mode, Y, nullptr, nullptr, s, colsq, formed);
+  return ttmc_impl(c, mode, Y, nullptr, nullptr, nullptr, s, colsq, formed);
 }
 
-tucker_status launch_ttmc_ex(Ctx *c, int mode, float *Y, const float *val, const float *const *Uf, cudaStream_t s) {
-  return ttmc_impl(c, mode, Y, val, Uf, s);
+tucker_status launch_ttmc_ex(Ctx *c, int mode, float *Y, const float *val, const uint32_t *vsrc,
+                             const float *const *Uf, cudaStream_t s) {
+  return ttmc_impl(c, mode, Y, val, vsrc, Uf, s);
 }
 
 }  // namespace tk

@@ -31,7 +31,7 @@ static int tile_width(int c, int no) {  // kernel widths: 4, 5, 6, 7, 8; 7 only 
   return c;
 }
 
-static TileChoice tile_choose(int nother, const int *R /* slot order */, double len) {
+static TileChoice tile_choose(int nother, const int *R /* slot order */, double len, bool adj) {
   TileChoice best{0, 0, 0, 0, 1e300};
   int64_t lead = 1;
   for (int t = 2; t < nother; ++t) lead *= R[t];
@@ -45,6 +45,7 @@ static TileChoice tile_choose(int nother, const int *R /* slot order */, double 
       c.cB = hb ? 4 : lB.T;
       c.TA = nother > 1 ? tile_width(c.cA, nother) : 1;
       c.TB = tile_width(c.cB, nother);
+      if (adj && !tile_adj_covers(c.TA, c.TB, nother)) continue;
       const int nA = lA.n * (ha ? 2 : 1), nB = lB.n * (hb ? 2 : 1);
       const int64_t G = lead * nA * nB;
       const int Gw = (int)std::min<int64_t>(G, 32), NG = 32 / Gw;
@@ -56,6 +57,7 @@ static TileChoice tile_choose(int nother, const int *R /* slot order */, double 
       const double passes = std::max(1.0 + slices, 32.0 / NG + 0.5 * (1.0 + slices));
       const double flush = slices * (20.0 + c.TA * (8.0 + (Gw * c.TB + 31) / 32 * (10.0 + 2.0 * NG)));
       c.cost = blocks * (passes * std::max(slots, lds) + flush + 40.0) * (1.0 + 3.0 / tile_min_blocks(tile));
+      if (adj && G > 32) continue;
       if (c.cost < best.cost) best = c;
     }
   return best;
@@ -81,23 +83,22 @@ static cudaError_t tile_dispatch_12(int TA, int TB, TileParams &p, int num_sms, 
   }
 }
 
-cudaError_t launch_ttmc_tile(const TileCall &c, cudaStream_t s) {
-  TileParams p{};
+static TileChoice tile_plan(const TileCall &c, bool adj, TileParams &p) {
   const int no = c.nother;
   p.nother = no;
-  int RS = 0;
+  int used = 0;
   for (int t = 0; t < no; ++t) {  // slots: the remaining modes backwards
     const int m = no - 1 - t;
     const int row = tile_layout(c.R[m]).row();
     p.idx[t] = c.idx[m];
     p.U[t] = c.U[m];
     p.R[t] = c.R[m];
-    p.off[t] = RS;
+    p.off[t] = used;
     for (p.lq[t] = 0; (4 << p.lq[t]) < row; ++p.lq[t]) {
     }
-    RS += row;
+    used += row;
   }
-  const TileChoice k = tile_choose(no, p.R, c.slice_len);
+  const TileChoice k = tile_choose(no, p.R, c.slice_len, adj);
   const TileLayout lB = tile_layout(p.R[0]);
   p.cB = k.cB;
   p.nB = k.cB == lB.T ? lB.n : 2 * lB.n;
@@ -113,8 +114,10 @@ cudaError_t launch_ttmc_tile(const TileCall &c, cudaStream_t s) {
   for (int t = 2; t < no; ++t) G *= p.R[t];
   p.G = (int)G;
   p.Gw = std::min(p.G, 32);
-  p.RS = 4 * tile_record(RS / 4, p.Gw, p.nB, p.nA, 1 << p.lq[0], no > 1 ? 1 << p.lq[1] : 1);
+  if (adj)  // a power of two
+    for (p.Gw = 1; p.Gw < p.G && p.Gw < 32;) p.Gw *= 2;
   p.NG = 32 / p.Gw;
+  p.RS = 4 * tile_record(used / 4, p.Gw, p.nB, p.nA, 1 << p.lq[0], no > 1 ? 1 << p.lq[1] : 1);
   p.val = c.val;
   p.vsrc = c.vsrc;
   p.sptr = c.sptr;
@@ -128,7 +131,76 @@ cudaError_t launch_ttmc_tile(const TileCall &c, cudaStream_t s) {
   p.Y = c.Y;
   p.carry = c.carry;
   p.P = c.P;
-  return no <= 2 ? tile_dispatch_12(k.TA, k.TB, p, c.num_sms, s) : tile_dispatch_n(k.TA, k.TB, p, c.num_sms, s);
+  return k;
+}
+
+cudaError_t launch_ttmc_tile(const TileCall &c, cudaStream_t s) {
+  TileParams p{};
+  const TileChoice k = tile_plan(c, false, p);
+  return c.nother <= 2 ? tile_dispatch_12(k.TA, k.TB, p, c.num_sms, s) : tile_dispatch_n(k.TA, k.TB, p, c.num_sms, s);
+}
+
+// ---- adjoint form
+// Q = U G_(n) in the order of the lanes' tiles: block = 128 places of a row (entry i of lane
+// j's tile at i * Gw + j, zero where there is none), some rows; the columns of G of those places
+// are held in shared memory.  Rows of U are read by all threads alike.
+constexpr int kQCols = 128, kQRows = 16;
+__global__ void __launch_bounds__(kQCols) tile_q_kernel(const TileParams p, const float *__restrict__ U,
+                                                        const float *__restrict__ G, int64_t I, int R, int TB, int QP,
+                                                        float *__restrict__ Q) {
+  extern __shared__ float gs[];  // [R][kQCols]
+  const int f = (int)blockIdx.y * kQCols + (int)threadIdx.x;
+  int64_t col = -1;
+  if (f < QP) {
+    const int i = f / p.Gw, j = f % p.Gw, a = i / TB, b = i % TB;
+    if (j < p.G && a < p.cA && b < p.cB) {
+      const int R1 = p.nother == 1 ? 1 : p.R[1], R0 = p.R[0];
+      const int r = j / p.nB % p.nA * (p.cA == 8 ? 4 : p.cA) + a + (a >= 4 ? p.jA : 0);
+      const int q = j % p.nB * (p.cB == 8 ? 4 : p.cB) + b + (b >= 4 ? p.jB : 0);
+      if (r < R1 && q < R0) col = ((int64_t)(j / p.nB / p.nA) * R1 + r) * R0 + q;
+    }
+  }
+  for (int r = 0; r < R; ++r) gs[r * kQCols + threadIdx.x] = col >= 0 ? __ldg(G + r * p.P + col) : 0.f;
+  if (f >= QP) return;
+  const int64_t i0 = (int64_t)blockIdx.x * kQRows, i1 = min(I, i0 + kQRows);
+  int64_t i = i0;
+  for (; i + 3 < i1; i += 4) {  // four rows at a time: their loads are in flight together
+    float t[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int r = 0; r < R; ++r) {
+      const float g = gs[r * kQCols + threadIdx.x];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) t[k] = fmaf(__ldg(U + (i + k) * R + r), g, t[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Q[(i + k) * QP + f] = t[k];
+  }
+  for (; i < i1; ++i) {
+    float t = 0.f;
+    for (int r = 0; r < R; ++r) t = fmaf(__ldg(U + i * R + r), gs[r * kQCols + threadIdx.x], t);
+    Q[i * QP + f] = t;
+  }
+}
+
+// The tile the adjoint form runs with, or false where a row has more tiles than a warp lanes.
+bool tile_adj_plan(const TileCall &c, int64_t *row_floats) {
+  TileParams p{};
+  const TileChoice k = tile_plan(c, true, p);
+  *row_floats = (int64_t)k.TA * k.TB * p.Gw;
+  return p.G <= 32 && k.cost < 1e300;
+}
+
+cudaError_t launch_tile_adj(const TileCall &c, const TileAdj &a, cudaStream_t s) {
+  TileParams p{};
+  const TileChoice k = tile_plan(c, true, p);
+  const int QP = k.TA * k.TB * p.Gw;
+  const dim3 grid((unsigned)((a.I + kQRows - 1) / kQRows), (unsigned)((QP + kQCols - 1) / kQCols));
+  tile_q_kernel<<<grid, kQCols, (size_t)a.R * kQCols * sizeof(float), s>>>(p, a.U, a.G, a.I, a.R, k.TB, QP, a.Q);
+  ::tk::count_launch();
+  p.Q = a.Q;
+  p.esrc = a.esrc;
+  p.e_out = a.e_out;
+  p.sq_part = a.sq_part;
+  return tile_dispatch_adj(k.TA, k.TB, p, c.num_sms, s);
 }
 
 // ---- factor copies in the tiled layout

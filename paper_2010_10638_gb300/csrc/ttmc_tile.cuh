@@ -33,6 +33,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "dfloat.cuh"
 #include "internal.cuh"
 
 namespace tk {
@@ -64,6 +65,11 @@ struct TileParams {
   int nA, nB;  // chunks of slots 1 and 0 (nA = 1 with one remaining mode)
   int cA, cB;  // ranks in a chunk
   int jA, jB;  // ranks skipped after the first four of a chunk
+  // adjoint form: the model's value is subtracted first, see tile_kernel
+  const float *Q;        // [I][TA * TB][Gw] rows of U_n G_(n) in the order of the lanes' tiles
+  const uint32_t *esrc;  // where the residual of sorted position e goes: e_out[esrc[e]], or e_out[e]
+  float *e_out;
+  double *sq_part;       // [n_units] sums of squared residuals
 };
 
 __device__ __forceinline__ void tile_cp16(uint32_t dst, const void *src) {
@@ -152,6 +158,32 @@ struct TileAcc {
       if constexpr (OB != 0) o[i] = fmaf(tile_unpack(sa).x, b[TB - 1], o[i]);
     }
   }
+  template <typename F>
+  __device__ __forceinline__ void load(F f) {  // entry i of the flat tile is f(i)
+#pragma unroll
+    for (int a = 0; a < TA; ++a) {
+#pragma unroll
+      for (int k = 0; k < PB; ++k) p[a * PB + k] = tile_pack(f(a * TB + 2 * k), f(a * TB + 2 * k + 1));
+      if constexpr (OB != 0) o[a] = f(a * TB + TB - 1);
+    }
+  }
+  __device__ __forceinline__ float dot(const float (&a)[TA], const float (&b)[TB]) const {  // a^T tile b
+    TileF2 b2[PB];
+#pragma unroll
+    for (int k = 0; k < PB; ++k) b2[k] = tile_pack(b[2 * k], b[2 * k + 1]);
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < TA; ++i) {
+      TileF2 t = tile_pack(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < PB; ++k) t = tile_fma2(p[i * PB + k], b2[k], t);
+      const float2 q = tile_unpack(t);
+      float r = q.x + q.y;
+      if constexpr (OB != 0) r = fmaf(o[i], b[TB - 1], r);
+      s = fmaf(a[i], r, s);
+    }
+    return s;
+  }
   __device__ __forceinline__ void row(int a, float (&v)[TB]) const {  // a known at compile time
 #pragma unroll
     for (int k = 0; k < PB; ++k) {
@@ -215,8 +247,15 @@ constexpr int tile_min_blocks(int tile) {  // blocks of 128 threads an SM is to 
 }
 
 // NO: remaining modes whose indices are held in registers (1, 2, 3, or 7 for 4 to 7).
-template <int NO, int TA, int TB>
-__global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB))
+//
+// ADJ (adjoint.cu): the TTMc of the residuals e_z = <Q(i_n, :), kron rows of z> - x_z, which it
+// forms on the way and writes out: a lane holds its tile of the slice's row of Q beside its
+// sums, so the gathers, which bound this kernel, are made once for both (10M observations,
+// ranks 10^3: 0.40 ms; one thread per nonzero forming e_z alone took 1.71 ms, and the TTMc
+// 0.30 ms after it).  A group's lanes add their parts of the inner product by shuffles (Gw a
+// power of two; all groups step together).
+template <int NO, int TA, int TB, bool ADJ>
+__global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB * (ADJ ? 2 : 1)))
     ttmc_tile_kernel(const __grid_constant__ TileParams p) {
   static_assert(NO > 1 || TA == 1, "one remaining mode: tiles of one row");
   constexpr unsigned kAll = 0xffffffffu;
@@ -293,6 +332,9 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB))
 
   TileAcc<TA, TB> acc;
   acc.clear();
+  TileAcc<TA, TB> qt;  // ADJ: this lane's tile of the slice's row of Q
+  bool fresh = true;   //      not loaded yet
+  DF sq;
   uint32_t kb = __ldg(p.unit_k0 + u);
   uint32_t bound = (kb + 1u + lane <= p.S) ? __ldg(p.sptr + kb + 1u + lane) : 0xffffffffu;
   load_ids(0);
@@ -317,6 +359,8 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB))
       tile_wait<0>();
     }
     __syncwarp();
+    uint32_t eo = e + (uint32_t)lane;
+    if (ADJ && p.esrc && lane < nt) eo = __ldg(p.esrc + eo);
     const uint32_t st = ring_s + (uint32_t)((t & 1) * 32 * RS) * 4u;
     const uint32_t xs = ring_s + (uint32_t)(64 * RS + 32 * (t & 1)) * 4u;
     uint32_t segs = starts | 1u;
@@ -325,7 +369,37 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB))
       const int p0 = __ffs(segs) - 1;
       segs &= segs - 1u;
       const int p1 = segs ? (__ffs(segs) - 1) : nt;
-      if (g < NG) {
+      if constexpr (ADJ) {
+        if (fresh) {
+          const float *Q = p.Q + (size_t)__ldg(p.sid + kseg) * (size_t)(TA * TB * Gw) + lane % Gw;
+          qt.load([&](int i) { return __ldg(Q + i * Gw); });
+          fresh = false;
+        }
+        for (int z0 = p0; z0 < p1; z0 += NG) {
+          const int z = min(z0 + g, p1 - 1);  // past the slice: its last position, with no residual
+          const uint32_t rec = st + (uint32_t)(z * RS) * 4u;
+          float lead_s = 1.f;
+          if constexpr (NO > 2) {
+#pragma unroll
+            for (int m = 2; m < NO; ++m)
+              if (m < nother) lead_s *= tile_lds1(rec + loff[m - 2]);
+          }
+          float av[TA], bv[TB];
+          if constexpr (NO == 1)
+            av[0] = 1.f;
+          else
+            tile_lds<TA>(rec + aoff, hopA, av);
+          tile_lds<TB>(rec + boff, hopB, bv);
+          const float x = tile_lds1(xs + (uint32_t)z * 4u);
+          float xhat = lead_s * qt.dot(av, bv);
+          for (int o = 1; o < Gw; o <<= 1) xhat += __shfl_xor_sync(kAll, xhat, o);
+          const bool in = z0 + g < p1;
+          const float r = in ? xhat - x : 0.f;
+          acc.add(lead_s * r, av, bv);
+          // (its value is no longer read: groups past the slice ignore what they read there)
+          if (in && lane % Gw == 0) asm volatile("st.shared.f32 [%0], %1;" ::"r"(xs + (uint32_t)z * 4u), "f"(r) : "memory");
+        }
+      } else if (g < NG) {
         const uint32_t rec = st + (uint32_t)((p0 + g) * RS) * 4u, adv = (uint32_t)(NG * RS) * 4u;
         uint32_t at_x = xs + (uint32_t)(p0 + g) * 4u, at_a = rec + aoff, at_b = rec + boff;
         uint32_t at_l[NO > 2 ? NO - 2 : 1];
@@ -387,19 +461,34 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB))
           __syncwarp();
         }
         acc.clear();
+        fresh = true;
       }
       ++kseg;
     }
     __syncwarp();
+    if constexpr (ADJ) {
+      if (lane < nt) {
+        const float r = tile_lds1(xs + (uint32_t)lane * 4u);
+        p.e_out[eo] = r;
+        df_fma(sq, r, r, 0.f);
+      }
+      __syncwarp();  // read before the next step's values are copied there
+    }
     kb = kb_next;
+  }
+  if constexpr (ADJ) {
+    double s = (double)sq.hi + (double)sq.lo;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kAll, s, o);
+    if (lane == 0) p.sq_part[u] = s;
   }
 }
 
 constexpr size_t kTileSmem = 227 * 1024;  // shared memory a block may have
 
-template <int NO, int TA, int TB>
+template <int NO, int TA, int TB, bool ADJ = false>
 static cudaError_t run_tile(TileParams &p, int num_sms, cudaStream_t s) {
-  auto kern = ttmc_tile_kernel<NO, TA, TB>;
+  auto kern = ttmc_tile_kernel<NO, TA, TB, ADJ>;
   const size_t per = (size_t)tile_warp_floats(p.RS, TB) * sizeof(float);
   const int most = (int)std::min<size_t>(kTileWarps, kTileSmem / per);
   if (most < 1) return cudaErrorInvalidConfiguration;
@@ -413,6 +502,8 @@ static cudaError_t run_tile(TileParams &p, int num_sms, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t tile_dispatch_n(int TA, int TB, TileParams &p, int num_sms, cudaStream_t s);  // ttmc_tile_n.cu
+cudaError_t tile_dispatch_n(int TA, int TB, TileParams &p, int num_sms, cudaStream_t s);    // ttmc_tile_n.cu
+cudaError_t tile_dispatch_adj(int TA, int TB, TileParams &p, int num_sms, cudaStream_t s);  // ttmc_tile_adj.cu
+bool tile_adj_covers(int TA, int TB, int nother);
 
 }  // namespace tk
