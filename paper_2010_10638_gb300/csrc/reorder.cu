@@ -361,9 +361,72 @@ __global__ void __launch_bounds__(kCpThreads) tile_compact_kernel(ChangePred pre
   if (sent && blockIdx.x == 0 && threadIdx.x == 0) sent[*sent_idx] = sent_val;
 }
 
+// Sum of the values of the group of equal coordinates that starts at position e, by a whole
+// warp: 128 positions a step, all loads of a step in flight.  The result is that of adding the
+// values one after another in FP64 from zero, in any case: where every value is a multiple of
+// 2^q and no sum of them reaches 2^(q + 53), FP64 additions are exact and their order does not
+// matter, which the largest and smallest exponent and the count tell; else they are added in
+// order (a chain of dependent additions, 64 cycles each here).  One thread that compared and
+// added one position at a time took 1.2 ms over the largest group (some 2,500 entries) of 1M
+// Zipf(1.1)^3 coordinates; the kernel now takes 0.02 ms.
+__device__ __forceinline__ double group_sum(const ChangePred &p, const float *vals, int64_t e, int lane) {
+  constexpr int kU = 4;
+  double part = 0.0;
+  uint32_t hi = 0u, lo = 0xffffffffu;
+  int64_t cur = e, end = -1;
+  while (end < 0) {
+    bool same[kU];
+    float v[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int64_t q = cur + 32 * u + lane;
+      v[u] = q < p.n ? __ldg(vals + q) : 0.f;
+      bool eq = q < p.n;
+      if (eq && q > e)
+        for (int m = 0; m < p.nw; ++m) eq = eq && __ldg(p.w[m] + q) == __ldg(p.w[m] + q - 1);
+      same[u] = eq;
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const unsigned out = ~__ballot_sync(0xffffffffu, same[u]);
+      if (end >= 0) continue;
+      const int cnt = out ? __ffs(out) - 1 : 32;
+      if (lane < cnt) {
+        part += (double)v[u];
+        const uint32_t x = (__float_as_uint(v[u]) >> 23) & 0xffu;  // (values are finite)
+        if (v[u] != 0.f) {
+          hi = max(hi, x);
+          lo = min(lo, max(x, 1u));
+        }
+      }
+      if (cnt < 32) end = cur + 32 * u + cnt;
+    }
+    cur += 32 * kU;
+  }
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  const int64_t n = end - e;
+  const int bits = (int)hi - (int)min(lo, hi) + 24 + (64 - __clzll(n));  // of a sum, above its last place
+  if (bits <= 53) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    return part;
+  }
+  double sum = 0.0;
+  for (int64_t q = e; q < end; q += 32) {
+    const float v = q + lane < end ? __ldg(vals + q + lane) : 0.f;
+    const int cnt = (int)min((int64_t)32, end - q);
+    for (int k = 0; k < cnt; ++k) sum += (double)__shfl_sync(0xffffffffu, v, k);
+  }
+  return sum;
+}
+
 // One group of equal coordinates -> one nonzero at its rank: FP64 sum of its values in sorted
 // (= input, the sort being stable) order; the squares of the sums, per tile, into part[tile].
 // Coordinate m of sorted position e is pred.w[m][e]; a run start of pred is a group head.
+// A group's end comes from the ballots; up to kCoSerial values are added by the head's lane,
+// longer groups (and those that go on past the warp's positions) by the warp.
+constexpr int kCoSerial = 32;
 __global__ void __launch_bounds__(kCpThreads, 1) coalesce_write_kernel(ChangePred pred, const float *vals,
                                                                    const uint32_t *prefix, int64_t nout,
                                                                    uint32_t *out_coords, float *out_vals,
@@ -371,7 +434,7 @@ __global__ void __launch_bounds__(kCpThreads, 1) coalesce_write_kernel(ChangePre
   __shared__ uint32_t woff[kCpWarps];
   __shared__ double wsq[kCpWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t e0 = (int64_t)blockIdx.x * kCpTile + w * (kCpSteps * 32) + lane;
+  const int64_t w0 = (int64_t)blockIdx.x * kCpTile + w * (kCpSteps * 32), e0 = w0 + lane;
   const int64_t n = pred.n;
   uint32_t bal[kCpSteps];
   change_ballots(pred, e0, lane, bal);
@@ -388,6 +451,22 @@ __global__ void __launch_bounds__(kCpThreads, 1) coalesce_write_kernel(ChangePre
       r += (uint32_t)__popc(bal[j]);
     }
   }
+  // first group start in the steps after step j, counted from w0; past the warp's positions:
+  // their end where a group starts there (or the entries end), else not known
+  const int kOpen = 1 << 20;
+  int next[kCpSteps];
+  {
+    const int64_t ew = w0 + kCpSteps * 32;
+    bool fresh = ew >= n;
+    if (!fresh)
+      for (int m = 0; m < pred.nw; ++m) fresh = fresh || __ldg(pred.w[m] + ew) != __ldg(pred.w[m] + ew - 1);
+    int at = fresh ? (int)min((int64_t)kCpSteps * 32, n - w0) : kOpen;
+#pragma unroll
+    for (int j = kCpSteps - 1; j >= 0; --j) {
+      next[j] = at;
+      if (bal[j]) at = 32 * j + __ffs(bal[j]) - 1;
+    }
+  }
   float v[kCpSteps];
 #pragma unroll
   for (int j = 0; j < kCpSteps; ++j) v[j] = (e0 + j * 32 < n) ? __ldg(vals + e0 + j * 32) : 0.0f;
@@ -397,23 +476,20 @@ __global__ void __launch_bounds__(kCpThreads, 1) coalesce_write_kernel(ChangePre
   for (int j = 0; j < kCpSteps; ++j) {
     const uint32_t rank = r + (uint32_t)__popc(bal[j] & lt);
     r += (uint32_t)__popc(bal[j]);
-    if ((bal[j] >> lane) & 1u) {
-      const int64_t e = e0 + j * 32;
-      double sum = (double)v[j];
-      // the next position starts a group when its bit says so (lane 31 of the warp's last
-      // step looks at the positions after it directly)
-      bool next_head;
-      if (lane < 31) next_head = (bal[j] >> (lane + 1)) & 1u;
-      else if (j + 1 < kCpSteps) next_head = bal[j + 1] & 1u;
-      else next_head = false;
-      if (e + 1 < n && !next_head) {
-        for (int64_t e2 = e + 1; e2 < n; ++e2) {
-          bool same = true;
-          for (int m = 0; m < pred.nw; ++m) same = same && (pred.w[m][e2] == pred.w[m][e2 - 1]);
-          if (!same) break;
-          sum += (double)__ldg(vals + e2);
-        }
-      }
+    const bool head = (bal[j] >> lane) & 1u;
+    const uint32_t above = bal[j] & ~lt & ~(1u << lane);
+    const int len = (above ? 32 * j + __ffs(above) - 1 : next[j]) - (32 * j + lane);
+    double sum = (double)v[j];
+    if (head && len <= kCoSerial)
+      for (int q = 1; q < len; ++q) sum += (double)__ldg(vals + e0 + j * 32 + q);
+    unsigned big = __ballot_sync(0xffffffffu, head && len > kCoSerial);
+    while (big) {
+      const int src = __ffs(big) - 1;
+      big &= big - 1u;
+      const double s = group_sum(pred, vals, w0 + 32 * j + src, lane);
+      if (lane == src) sum = s;
+    }
+    if (head) {
       out_vals[rank] = (float)sum;
       acc += sum * sum;
     }
@@ -435,7 +511,7 @@ struct SliceWrite {
     const uint32_t i = __ldg(row + e);
     sptr[k] = (uint32_t)e;
     sid[k] = i;
-    present[i] = 1u;
+    if (present) present[i] = 1u;
   }
 };
 
@@ -601,6 +677,79 @@ __global__ void unit_count_kernel(int64_t S, const uint32_t *sptr, uint32_t chun
   }
 }
 
+// unit_count_kernel and the exclusive scans of both its lists in one block (total[0], total[1]:
+// their sums); up to kUnitScanMax slices, 4,096 a round (50,000 slices: 20 us as one launch,
+// against seven launches)
+constexpr int64_t kUnitScanMax = 1 << 16;
+__global__ void __launch_bounds__(1024) unit_scan_kernel(int64_t S, const uint32_t *__restrict__ sptr, uint32_t chunk,
+                                                         uint32_t run, uint32_t *__restrict__ nu,
+                                                         uint32_t *__restrict__ islong, uint32_t *__restrict__ uoff,
+                                                         uint32_t *__restrict__ lid, uint32_t *__restrict__ total) {
+  __shared__ unsigned long long wsum[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  unsigned long long carry = 0;  // units in the low word, long slices in the high one
+  for (int64_t k0 = 0; k0 < S; k0 += 4096) {
+    const int64_t b0 = k0 + 4 * (int64_t)threadIdx.x;
+    uint32_t at[6];  // sptr[b0 - 1 .. b0 + 4]
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const int64_t k = b0 - 1 + i;
+      at[i] = (k >= 0 && k <= S) ? __ldg(sptr + k) : 0u;
+    }
+    uint32_t n[4], l[4];
+    unsigned long long sum = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t k = b0 + i;
+      n[i] = l[i] = 0u;
+      if (k < S) {
+        const uint32_t b = at[i + 1], len = at[i + 2] - b, pb = at[i];
+        l[i] = len > chunk ? 1u : 0u;
+        const bool head = k == 0 || l[i] || b - pb > chunk || b / run != pb / run;
+        n[i] = l[i] ? (len + chunk - 1) / chunk : (head ? 1u : 0u);
+      }
+      sum += n[i] + ((unsigned long long)l[i] << 32);
+    }
+    unsigned long long incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) wsum[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+      const unsigned long long x = wsum[lane];
+      unsigned long long xi = x;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xffffffffu, xi, o);
+        if (lane >= o) xi += t;
+      }
+      wsum[lane] = xi;
+    }
+    __syncthreads();
+    unsigned long long off = carry + (w ? wsum[w - 1] : 0ull) + incl - sum;
+    carry += wsum[31];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t k = b0 + i;
+      if (k < S) {
+        nu[k] = n[i];
+        islong[k] = l[i];
+        uoff[k] = (uint32_t)off;
+        lid[k] = (uint32_t)(off >> 32);
+      }
+      off += n[i] + ((unsigned long long)l[i] << 32);
+    }
+    __syncthreads();  // wsum is read
+  }
+  if (threadIdx.x == 0) {
+    total[0] = (uint32_t)carry;
+    total[1] = (uint32_t)(carry >> 32);
+  }
+}
+
 __global__ void unit_write_kernel(int64_t S, const uint32_t *sptr, const uint32_t *nu,
                                   const uint32_t *uoff, const uint32_t *islong, const uint32_t *lid,
                                   uint32_t *unit_e0, uint32_t *unit_k0, int32_t *unit_slot, uint32_t *long_k,
@@ -718,10 +867,15 @@ static tucker_status build_units(Ctx *c, int64_t S, const uint32_t *ptr, UnitSiz
   const uint32_t chunk = (uint32_t)size.chunk, run = (uint32_t)size.run;
   uint32_t nunits = 0, nlong = 0;
   if (S > 0) {
-    unit_count_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, chunk, run, nu, islong);
-    ::tk::count_launch();
-    exclusive_scan_total(nu, uoff, S, stmp, d_small + 2, s);
-    exclusive_scan_total(islong, lid, S, stmp, d_small + 3, s);
+    if (S <= kUnitScanMax) {
+      unit_scan_kernel<<<1, 1024, 0, s>>>(S, ptr, chunk, run, nu, islong, uoff, lid, d_small + 2);
+      ::tk::count_launch();
+    } else {
+      unit_count_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, chunk, run, nu, islong);
+      ::tk::count_launch();
+      exclusive_scan_total(nu, uoff, S, stmp, d_small + 2, s);
+      exclusive_scan_total(islong, lid, S, stmp, d_small + 3, s);
+    }
     uint32_t h2[2];
     TK_TRY(cudaMemcpyAsync(h2, d_small + 2, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     TK_TRY(cudaStreamSynchronize(s));
@@ -785,6 +939,7 @@ cudaError_t preload_reorder_kernels() {
       reinterpret_cast<const void *>(fiber_slices_kernel),
       reinterpret_cast<const void *>(unit_fiber_kernel),
       reinterpret_cast<const void *>(unit_count_kernel),
+      reinterpret_cast<const void *>(unit_scan_kernel),
       reinterpret_cast<const void *>(unit_write_kernel),
       reinterpret_cast<const void *>(unit_long_kernel),
   };
@@ -990,24 +1145,21 @@ tucker_status build_sorted_copies(Ctx *c, const uint32_t *coords_in, const float
     mc.S = S;
     TK_TRY(dev_alloc(c, &mc.sptr, (size_t)S + 1));
     TK_TRY(dev_alloc(c, &mc.sid, (size_t)std::max<uint32_t>(S, 1)));
-    TK_TRY(cudaMemsetAsync(present, 0, sizeof(uint32_t) * (size_t)mc.I, s));
+    const int64_t ne = mc.I - (int64_t)S;  // empty rows
+    if (ne) TK_TRY(cudaMemsetAsync(present, 0, sizeof(uint32_t) * (size_t)mc.I, s));
     if (Z > 0) {
-      const SliceWrite sw{row, mc.sptr, mc.sid, present};
+      const SliceWrite sw{row, mc.sptr, mc.sid, ne ? present : nullptr};
       tile_compact_kernel<<<(unsigned)cp_tiles(Z), kCpThreads, 0, s>>>(rp, prefix, sw, mc.sptr, d_small, (uint32_t)Z);
       ::tk::count_launch();
     } else {
       TK_TRY(cudaMemsetAsync(mc.sptr, 0, sizeof(uint32_t), s));
     }
-    // empty rows
-    invert_flag_kernel<<<grid_for(mc.I), 256, 0, s>>>(mc.I, present, flag);
-    ::tk::count_launch();
-    exclusive_scan_total(flag, pos, mc.I, stmp, d_small + 1, s);
-    uint32_t ne = 0;
-    tucker_status st = read_u32(c, d_small + 1, &ne, s);
-    if (st != TUCKER_OK) return st;
     mc.n_empty = ne;
-    TK_TRY(dev_alloc(c, &mc.empty, (size_t)std::max<uint32_t>(ne, 1)));
+    TK_TRY(dev_alloc(c, &mc.empty, (size_t)std::max<int64_t>(ne, 1)));
     if (ne) {
+      invert_flag_kernel<<<grid_for(mc.I), 256, 0, s>>>(mc.I, present, flag);
+      ::tk::count_launch();
+      exclusive_scan_total(flag, pos, mc.I, stmp, nullptr, s);
       compact_kernel<<<grid_for(mc.I), 256, 0, s>>>(mc.I, flag, pos, mc.empty);
       ::tk::count_launch();
     }
@@ -1050,6 +1202,15 @@ tucker_status build_sorted_copies(Ctx *c, const uint32_t *coords_in, const float
     if (mc.S == 0) continue;
     int mid_mode = mc.other[0];  // modes 2, 3: mode 1
     bool resorted = false;
+    // The runs of (slice, middle index), at most as many as the fibers, are known already: the
+    // distinct (i_1, i_n) pairs, of the middle mode for mode 1.  More of them than fibers are
+    // wanted: no fiber level, no re-sort and none of the kernels and read-backs below.
+    if (fp != 1) {
+      const bool third = fnat[1] > 0 && fnat[2] > 0 && (double)fnat[2] <= 0.8 * (double)fnat[1];
+      const uint32_t runs = n > 0 ? fnat[n] : fnat[third ? 2 : 1];
+      if ((double)runs > kFiberShare * (double)Z && (n > 0 || (third ? 2 : 1) == mid0 || c->mode[third ? 2 : 1].src))
+        continue;
+    }
     if (n == 0) {
       mid_mode = (fnat[1] > 0 && fnat[2] > 0 && (double)fnat[2] <= 0.8 * (double)fnat[1]) ? 2 : 1;
       if (mid_mode != mid0 && rows[mid_mode] && c->mode[mid_mode].src) {

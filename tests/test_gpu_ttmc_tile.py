@@ -100,3 +100,50 @@ def test_adjoint_with_factors_at_any_address(ranks):
     L, dU, dG = T.tucker_loss_grad(ctx, Uf, G)
     L2, dU2, dG2 = T.tucker_loss_grad(ctx, odd, G)
     assert torch.equal(L, L2) and torch.equal(dG, dG2) and all(torch.equal(a, b) for a, b in zip(dU, dU2))
+
+
+def test_heavy_duplicates_sum_as_one_after_another():
+    """Groups of equal coordinates of every length around the warp's 32 and the tile's 512 and
+    8,192 positions: the values of the context are the FP64 sums in input order, rounded once, both
+    where those sums are exact in any order and where (exponents 100 apart) they are not."""
+    T = lib()
+    rng = np.random.default_rng(5)
+    lens = [1, 2, 31, 32, 33, 34, 127, 128, 129, 500, 512, 513, 2500, 8192, 9001, 1, 3]
+    for spread in (0, 50):
+        idx = np.concatenate([np.full(k, i) for i, k in enumerate(lens)])
+        rng.shuffle(idx)
+        vals = (rng.standard_normal(idx.size) * 2.0 ** rng.integers(-spread, spread + 1, idx.size)).astype(np.float32)
+        coords = np.stack([idx % 5, idx // 5]).astype(np.uint32)
+        ctx = T.tucker_init((5, 5), torch.as_tensor(coords.astype(np.int32)).cuda(), torch.as_tensor(vals).cuda(), (1, 1),
+                            [torch.ones((5, 1), dtype=torch.float64).cuda() for _ in range(2)])
+        want = np.zeros(25)
+        for i, v in zip(idx, vals.astype(np.float64)):
+            want[i] += v  # one after another
+        assert T.tucker_nnz(ctx) == len(lens)
+        np.testing.assert_allclose(T.tucker_norm2(ctx), (want ** 2).sum(), rtol=1e-14)
+        dense = np.zeros((5, 5))
+        dense.reshape(-1)[:] = 0
+        for i in range(len(lens)):
+            dense[i % 5, i // 5] = np.float32(want[i])
+        for j in range(5):  # one column at a time: its entries are the context's values themselves
+            e = torch.zeros((5, 1), dtype=torch.float64)
+            e[j] = 1.0
+            T.tucker_set_factor(ctx, 1, e.cuda())
+            np.testing.assert_array_equal(T.ttmc_mode(ctx, 0).cpu().numpy()[:, 0].astype(np.float64), dense[:, j])
+
+
+@pytest.mark.parametrize("rows", [4095, 4097, 70_000])
+def test_units_of_many_slices(rows):
+    """More slices than one round of the unit scan (4,096), and than its one block takes."""
+    T = lib()
+    rng = np.random.default_rng(rows)
+    k = rng.integers(1, 4, rows)
+    k[[0, rows // 2, rows - 1]] = 700  # cut slices at the ends
+    i0 = np.repeat(np.arange(rows), k)
+    coords = np.stack([i0, rng.integers(0, 50, i0.size), rng.integers(0, 60, i0.size)]).astype(np.uint32)
+    vals = rng.standard_normal(i0.size).astype(np.float32)
+    dims, ranks = (rows, 50, 60), (2, 3, 5)
+    U = [rng.standard_normal((d, r)) for d, r in zip(dims, ranks)]
+    ctx = T.tucker_init(dims, torch.as_tensor(coords.astype(np.int32)).cuda(), torch.as_tensor(vals).cuda(), ranks,
+                        [torch.as_tensor(u).cuda() for u in U])
+    check(T, ctx, dims, ranks, coords, vals, f32_round(U))
