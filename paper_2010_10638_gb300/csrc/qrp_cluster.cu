@@ -670,8 +670,23 @@ __device__ void ccolsum(const CArgs &a, const AT *As, int64_t ncache, int64_t r0
       const int64_t c = c0 + cl;
       double acc = 0.0;
       if (act && c < n) {
-        for (int64_t li = l0 + rl; li < nrows; li += nrl) {
-          const double x = li < ncache ? (double)As[li * n + c] : (double)__ldg(A + (r0 + li) * a.lda + c);
+        int64_t li = l0 + rl;
+        for (; li < min(nrows, ncache); li += nrl) {
+          const double x = (double)As[li * n + c];
+          acc = fma(x, SQUARE ? x : yd[li], acc);
+        }
+        // rows in global memory, eight loads in flight: with one row at a time a thread waited
+        // out the latency of L2 for each (20,000 x 256, k = 16: 580 us, 36 us a reflector, of
+        // which the FP64 pipe needs 8)
+        for (; li + 7 * nrl < nrows; li += 8 * nrl) {
+          double x[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) x[u] = (double)__ldg(A + (r0 + li + u * nrl) * a.lda + c);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) acc = fma(x[u], SQUARE ? x[u] : yd[li + u * nrl], acc);
+        }
+        for (; li < nrows; li += nrl) {
+          const double x = (double)__ldg(A + (r0 + li) * a.lda + c);
           acc = fma(x, SQUARE ? x : yd[li], acc);
         }
       }
