@@ -216,6 +216,14 @@ static tucker_status init_impl(Ctx *c, const uint32_t *coords, const float *vals
     TK_CUDA(cudaMemsetAsync(c->sq_cnt, 0, 8 * sizeof(unsigned), s));
     c->sq_elems = rows;
   }
+  for (int n = 0; n < N; ++n)
+    if (qrp_n_cols(c, n) == c->mode[n].P)
+      c->qgram_bytes = std::max(c->qgram_bytes, qrp_gram_bytes(c->mode[n].I, c->mode[n].P, c->ranks[n], c->num_sms));
+  if (c->qgram_bytes && dev_alloc(c, &c->qgram, c->qgram_bytes) != cudaSuccess) {  // not needed: the cluster form
+    cudaGetLastError();
+    c->qgram = nullptr;
+    c->qgram_bytes = 0;
+  }
   TK_CUDA(dev_alloc(c, &c->G, (size_t)PR));
   TK_CUDA(dev_alloc(c, &c->core_part, core_part_elems(c->num_sms, c->mode[N - 1].P, c->ranks[N - 1])));
   TK_CUDA(dev_alloc(c, &c->core_counter, 4));
@@ -308,6 +316,8 @@ static tucker_status hooi_impl(Ctx *c, double *fit_out, cudaStream_t s) {
       st = qrp_run_f64(c->gram, mc.I, mc.I, mc.I, k, c->U64[n], k, nullptr, nullptr, &w, c->num_sms, s);
     } else {
       if (norms) w.colsq = c->colsq;
+      w.gram_ws = c->qgram;
+      w.gram_bytes = c->qgram_bytes;
       st = qrp_run_f32(c->Y, mc.I, mc.P, mc.P, k, c->U64[n], k, nullptr, nullptr, &w, c->num_sms, s);
     }
     if (st != TUCKER_OK) return st;

@@ -11,6 +11,7 @@
 #include <cstdlib>
 
 #include "internal.cuh"
+#include "tc.cuh"
 
 namespace tk {
 
@@ -102,7 +103,6 @@ constexpr int kTcKC = kTcK * 2 / 16;  // core-matrix columns (16 bytes) along K 
 constexpr int kTcRows = 128;  // rows of Y per CTA at most: keeps every level sum below 2^24
 constexpr int kTcSlices = 4;  // 8-bit slices per value
 constexpr int kTcLevels = 5;  // slice pairs a + b <= 4 (the three pairs above add under 2^-40 of a product)
-constexpr unsigned long long kTcSpin = 1ull << 22;
 
 __host__ __device__ constexpr uint32_t tc_tmem_cols(int np) {
   uint32_t c = 32;
@@ -116,13 +116,6 @@ __host__ __device__ constexpr size_t tc_smem_bytes(int rows, int np) {
   return tc_rows_bytes(rows, np) + (size_t)2 * kTcSlices * (kTcM + np) * kTcK * 2 + 128;  // + two slice buffers
 }
 
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;  // descriptor version of this architecture; base offset 0, no swizzle
-  return d;
-}
 // The four integer slices of an FP32 y against 2^e (|y| < 2^e; 2^(8 - e) = sc1 sc2, two
 // factors so that neither overflows when the column holds only subnormal values), each
 // exact in BF16.  FP32 arithmetic, all exact: t = y 2^(8 - e) has at most 24 significant
@@ -169,13 +162,7 @@ __device__ __forceinline__ void slices_f64(double u, int e, __nv_bfloat16 *out, 
 #pragma unroll
   for (int q = 0; q < kTcSlices; ++q) out[q * stride] = __int2bfloat16_rn(m[q]);
 }
-// exponent e with |x| < 2^e (0 for x = 0) of a finite FP32 / FP64 magnitude given by its bits
-// (the exponent field, or the leading zeros of a subnormal's fraction): integer arithmetic
-__device__ __forceinline__ int above_exp_f32(uint32_t b) {
-  const int ef = (int)(b >> 23);
-  if (ef) return ef - 126;
-  return b ? -149 + 32 - __clz((int)b) : 0;
-}
+// exponent e with |x| < 2^e of a finite FP64 magnitude given by its bits, as above_exp_f32
 __device__ __forceinline__ int above_exp_f64(unsigned long long b) {
   const int ef = (int)(b >> 52);
   if (ef) return ef - 1022;
@@ -187,21 +174,6 @@ __device__ __forceinline__ double pow2d(int k) { return __longlong_as_double((lo
 __device__ __forceinline__ int kmaj16(int row, int k) {
   return ((row >> 3) * kTcKC + (k >> 3)) * 64 + (row & 7) * 8 + (k & 7);
 }
-// bounded wait for completion `parity` of an mbarrier; false if it gave up
-__device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity) {
-  for (unsigned long long it = 0; it < kTcSpin; ++it) {
-    uint32_t d;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-        : "=r"(d)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (d) return true;
-    if (it > 32) __nanosleep(64);
-  }
-  return false;
-}
-
 template <int NP>  // N of the MMA: R rounded up to 16
 __global__ void __launch_bounds__(128) core_tc_kernel(const float *Y, const double *U, int64_t I, int64_t P, int R,
                                                       int rows_per_split, double *part, uint32_t *err) {

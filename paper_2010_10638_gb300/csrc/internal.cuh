@@ -89,6 +89,12 @@ struct QrpWork {
   // [n] column sums of squares of A given by the caller (FP32 A), or nullptr: the cluster
   // form then skips its own first pass over A and takes these as the initial norms
   const double *colsq = nullptr;
+  // FP32 A: workspace of the Gram form (qrp_gram.cu), or nullptr: not tried
+  void *gram_ws = nullptr;
+  size_t gram_bytes = 0;
+  // the cluster form runs only if this device word is not zero (nullptr: always)
+  const uint32_t *only_if = nullptr;
+  bool plan_only = false;  // the cluster form answers whether it takes the shape, and launches nothing
   size_t bytes = 0;
 };
 
@@ -146,6 +152,8 @@ struct Ctx {
   int sweeps = 0;
 
   QrpWork qw;
+  void *qgram = nullptr;       // workspace of the QRP's Gram form, for the largest mode
+  size_t qgram_bytes = 0;
   uint32_t *d_err = nullptr;   // latched device error bits
 
   bool profiling = false;      // record CUDA events around the phases of hooi_iter
@@ -314,6 +322,11 @@ void qrp_bind_work(QrpWork *w, void *base, int64_t m, int64_t n, int k, int nb);
 template <typename AT>
 bool qrp_cluster(const AT *A, int64_t m, int64_t n, int64_t lda, int k, double *Q, int64_t ldq, int64_t *piv,
                  double *rdiag, QrpWork *w, cudaStream_t s, cudaError_t *err);
+// Gram form (qrp_gram.cu): launches it and returns the device word that is not zero when it gave up
+const uint32_t *qrp_gram(const float *A, int64_t m, int64_t n, int64_t lda, int k, double *Q, int64_t ldq, QrpWork *w,
+                         int num_sms, cudaStream_t s, cudaError_t *err);
+bool qrp_gram_takes(int64_t m, int64_t n, int k, const QrpWork *w, int num_sms);  // the shape, with w's workspace
+size_t qrp_gram_bytes(int64_t m, int64_t n, int k, int num_sms);  // its workspace (0: not for this shape)
 tucker_status qrp_run_f64(const double *A, int64_t m, int64_t n, int64_t lda, int k, double *Q, int64_t ldq,
                           int64_t *piv, double *rdiag, QrpWork *w, int nb, cudaStream_t s);
 tucker_status qrp_run_f32(const float *A, int64_t m, int64_t n, int64_t lda, int k, double *Q, int64_t ldq,

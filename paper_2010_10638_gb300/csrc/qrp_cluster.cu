@@ -94,6 +94,7 @@ struct CArgs {
   int64_t ldq;
   int64_t *piv;
   double *rdiag;
+  const uint32_t *only_if;  // run only if this word is not zero (nullptr: always)
   const double *colsq;  // [n] column sums of squares of A given by the caller (FP32 A read as
                         // float4 only), or nullptr: the first pass over A forms them
 };
@@ -180,25 +181,11 @@ __device__ __forceinline__ void cp_async_elem(T *dst, const T *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
 }
 
-// double-float addition a += b (TwoSum of the high parts, then renormalisation)
-__device__ __forceinline__ void df_add(DF &a, const DF b) {
-  const float s = a.hi + b.hi;
-  const float bp = s - a.hi;
-  float e = (a.hi - (s - bp)) + (b.hi - bp);
-  e += a.lo + b.lo;
-  a.hi = s + e;
-  a.lo = e - (a.hi - s);
-}
-
 // Entries of the reductions' partial vectors.  FP32 A: double-float pairs (x = hi,
 // y = lo), so that their sums over the blocks of a cluster and over the clusters run on
 // the FP32 pipe (the FP64 pipe issues one warp instruction per 16 cycles per SM here),
 // with about 2^-48 relative error per addition; each needed entry is converted to FP64
 // once at the end.  FP64 A (values of any FP64 magnitude): FP64.
-__device__ __forceinline__ float2 df2_of(double v) {
-  const float h = __double2float_rn(v);
-  return make_float2(h, __double2float_rn(v - (double)h));
-}
 __device__ __forceinline__ double df2_val(float2 p) { return (double)p.x + (double)p.y; }
 __device__ __forceinline__ float2 df2_add(float2 a, float2 b) {
   DF x;
@@ -209,32 +196,6 @@ __device__ __forceinline__ float2 df2_add(float2 a, float2 b) {
   y.lo = b.y;
   df_add(x, y);
   return make_float2(x.hi, x.lo);
-}
-
-// t -= (v.x + v.y) (m.x + m.y): the product of the high parts exactly (FMA residual), the
-// cross terms by FMA, the low-low term dropped (2^-48 of the product); TwoSum of the high parts
-__device__ __forceinline__ void df_sub_prod(DF &t, float2 v, float2 m) {
-  const float p = v.x * m.x;
-  float e = fmaf(v.x, m.x, -p);
-  e = fmaf(v.x, m.y, e);
-  e = fmaf(v.y, m.x, e);
-  const float s = t.hi - p;
-  const float bp = s - t.hi;
-  const float err = (t.hi - (s - bp)) - (p + bp);
-  t.hi = s;
-  t.lo += err - e;
-}
-
-// FP32 -> FP64 without the FP64 pipe: the same sign, the exponent rebiased (+896), the
-// mantissa shifted up 29 bits; exact for normal numbers (zero, subnormals, inf and NaN
-// take the conversion instruction)
-__device__ __forceinline__ double f2d_exact(float f) {
-  const unsigned b = __float_as_uint(f);
-  const unsigned e = (b >> 23) & 0xffu;
-  if (e == 0u || e == 0xffu) return (double)f;
-  const unsigned long long d = ((unsigned long long)(b & 0x80000000u) << 32) |
-                               ((unsigned long long)(e + 896u) << 52) | ((unsigned long long)(b & 0x7fffffu) << 29);
-  return __longlong_as_double((long long)d);
 }
 
 template <typename PT>
@@ -817,6 +778,7 @@ __global__ void __launch_bounds__(kCT, 1) qrp_cluster_kernel(CArgs a) {
   __shared__ double s_f[64];  // F[p, 0:j] of the current pivot column
   __shared__ double s_sc[4];  // v_jj, tau, v_jj - y_jj
   __shared__ int s_ok, s_res;
+  if (a.only_if && *a.only_if == 0u) return;  // (the same word for every block)
   cg::cluster_group cl = cg::this_cluster();
   Team tm;
   tm.S = cl.num_blocks();
@@ -1333,6 +1295,7 @@ bool qrp_cluster(const AT *A, int64_t m, int64_t n, int64_t lda, int k, double *
   const size_t smem = need(S, rows_per, rows_cached);
   if (C > 1 && 2 * (size_t)C * L > w->part_elems) return false;  // the cluster sums live in `part`
   if ((int64_t)((C + 15) / 16) * ((n + S - 1) / S + 2 * k + 2) > 2 * kCT) return false;  // chunk sums: scratch
+  if (w->plan_only) return true;
 
   CArgs a{};
   a.A = A;
@@ -1358,6 +1321,7 @@ bool qrp_cluster(const AT *A, int64_t m, int64_t n, int64_t lda, int k, double *
   a.piv = piv;
   a.rdiag = rdiag;
   a.colsq = (es == 4 && a.vec4) ? w->colsq : nullptr;
+  a.only_if = w->only_if;
   if (C > 1 && (*err = cudaMemsetAsync(w->bar, 0, 3 * sizeof(unsigned), s)) != cudaSuccess) return true;
 
   cudaLaunchConfig_t cfg = {};
