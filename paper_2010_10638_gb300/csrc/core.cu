@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <cstdlib>
 
+#include "dfloat.cuh"
 #include "internal.cuh"
 #include "tc.cuh"
 
@@ -402,212 +403,101 @@ __global__ void __launch_bounds__(kRedT) core_reduce_kernel(const double *part, 
 
 static bool core_on_tensor_cores();
 
-// ---------------------------------------------------------------- Gram matrix on the tensor cores
-// S = Y Y^T (m x m) of an FP32 m x n matrix, for the fat unfoldings of Section III-D, with
-// the exact fixed-point slices of the core: one CTA computes a 128 x 64 tile of S (rows i
-// of Y as the MMA's M, rows j as its N) over a range of columns c (the K), 128 columns at
-// a time.  For each 128-column block every row of Y gets a shared power of two over the
-// block, the slices' level sums are exact integers in tensor memory (products <= 2^16, at
-// most 128 columns), and after each block they are combined in 64-bit integers and added,
-// scaled, into FP64 registers.  The column ranges are added in a fixed order afterwards.
-constexpr int kGmM = 128;           // rows i per tile (MMA M)
-constexpr int kGmN = 64;            // rows j per tile (MMA N)
-constexpr int kGmCols = 128;        // columns per exact block
-constexpr int kGmLd = kGmCols + 1;  // shared-memory row stride of the staged block (no bank conflicts)
-constexpr int kGramMaxRows = 1024;  // larger Gram matrices use the FP64 form
+// ---------------------------------------------------------------- Gram matrix of fat unfoldings
+// S = Y Y^T (m x m) of an FP32 m x n matrix (Section III-D, P_n > I_n): a 32 x 32 tile of S on and
+// below the diagonal over a range of columns, a 2 x 2 piece a thread.  32 columns at a time, every
+// row scaled by the power of two of its largest entry there (any magnitude of FP32 goes), exact
+// products are added in double-float (2^-46 of |y_i| |y_j|) and these sums in FP64; both triangles
+// are written, and the ranges added in order.
+// The FP32 pipe bounds it (11 instructions a product, half of the products by symmetry).  The
+// tensor cores on exact 8-bit slices (error 2^-33) took longer at every size, most of it in
+// slicing and hand-overs: 200 x 256 32 -> 11 us with the sum of the ranges; with the QRP that
+// follows 64 x 3,600 288 -> 191, 200 x 1,280 151 -> 104, 1,000 x 1,056 708 -> 652, 1,000 x 4,096
+// 1,682 -> 1,599.
+constexpr int kGramMaxRows = 1024;  // above, tiles alone fill the GPU: one range
 constexpr int kGramMaxRanges = 8;   // column ranges (partial sets)
-
-__host__ __device__ constexpr size_t gm_smem_bytes() {
-  return (size_t)(kGmM + kGmN) * kGmLd * 4                                // the rows' column block
-         + (size_t)2 * kTcSlices * (kGmM + kGmN) * kTcK * 2 + 128;        // two slice buffers
-}
-
-__global__ void __launch_bounds__(128) gram_tc_kernel(const float *Y, int64_t m, int64_t n, int64_t cols_per_range,
-                                                      double *part, uint32_t *err) {
-  constexpr uint32_t kCols = tc_tmem_cols(kGmN);
-  constexpr int kASlice = kGmM * kTcK, kBSlice = kGmN * kTcK;
-  extern __shared__ unsigned char gm_raw[];
-  unsigned char *base = reinterpret_cast<unsigned char *>(
-      (reinterpret_cast<uintptr_t>(gm_raw) + 127) & ~static_cast<uintptr_t>(127));
-  float *sYa = reinterpret_cast<float *>(base);  // [kGmM][kGmLd]: rows i of the block
-  float *sYb = sYa + kGmM * kGmLd;               // [kGmN][kGmLd]: rows j
-  __nv_bfloat16 *sA = reinterpret_cast<__nv_bfloat16 *>(
-      base + ((size_t)(kGmM + kGmN) * kGmLd * 4 + 127) / 128 * 128);
-  __nv_bfloat16 *sB = sA + 2 * kTcSlices * kASlice;
-  __shared__ __align__(8) unsigned long long bar[2];
-  __shared__ uint32_t tbase;
-  __shared__ int s_ok;
-  __shared__ int s_eb[kGmN];
-  __shared__ float s_bsc[2][kGmN];
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int64_t i0 = (int64_t)blockIdx.x * kGmM, j0 = (int64_t)blockIdx.y * kGmN;
-  const int64_t c_begin = (int64_t)blockIdx.z * cols_per_range;
-  const int64_t c_end = min(n, c_begin + cols_per_range);
-  uint32_t sb[2];
-  sb[0] = (uint32_t)__cvta_generic_to_shared(&bar[0]);
-  sb[1] = (uint32_t)__cvta_generic_to_shared(&bar[1]);
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sb[0]) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sb[1]) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    s_ok = 1;
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     (uint32_t)__cvta_generic_to_shared(&tbase)),
-                 "r"(kCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tbase;
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kGmN >> 3) << 17) | ((uint32_t)(kGmM >> 4) << 24);
-  const uint32_t lbo = 128, sbo = kTcKC * 128;
-  const uint32_t aS = (uint32_t)__cvta_generic_to_shared(sA), bS = (uint32_t)__cvta_generic_to_shared(sB);
-  const int64_t ri = i0 + tid;  // this thread's row i (TMEM lane)
-  double accd[kGmN];
+constexpr int kGdT = 32, kGdK = 32, kGdLd = kGdK + 4;
+__global__ void __launch_bounds__(256) gram_df_kernel(const float *__restrict__ Y, int m, int64_t n,
+                                                      int64_t cols_per_range, double *__restrict__ out) {
+  __shared__ __align__(16) float sa[kGdT][kGdLd], sb[kGdT][kGdLd];
+  __shared__ int ea[kGdT], eb[kGdT];  // the rows' exponents
+  int ti = 0, tj = (int)blockIdx.x;
+  while (tj > ti) tj -= ++ti;
+  const int i0 = ti * kGdT, j0 = tj * kGdT, tid = threadIdx.x;
+  const int64_t c_begin = (int64_t)blockIdx.y * cols_per_range, c_end = min(n, c_begin + cols_per_range);
+  const int ia = tid / 16, jb = tid % 16;  // rows ia, ia + 16 of the tile, columns jb, jb + 16
+  constexpr int kU = kGdT * kGdK / 256;
+  float va[kU], vb[kU];
+  auto load = [&](int64_t c0) {
 #pragma unroll
-  for (int q = 0; q < kGmN; ++q) accd[q] = 0.0;
-  bool ok = true;
-  int phase[2] = {0, 0};  // completions waited for, per buffer
-  int issued[2] = {0, 0};  // products issued, per buffer
-  int jglob = 0;           // chunk counter over all blocks (buffer = jglob & 1)
-  for (int64_t cb = c_begin; cb < c_end && ok; cb += kGmCols) {
-    const int ncb = (int)min((int64_t)kGmCols, c_end - cb);
-    const int nch = (ncb + kTcK - 1) / kTcK;
-    // the block's columns of rows i and rows j, zero-padded (coalesced along the rows)
-#pragma unroll 8
-    for (int q = tid; q < kGmM * kGmCols; q += 128) {
-      const int r = q / kGmCols, k = q % kGmCols;
-      const int64_t rr = i0 + r;
-      sYa[r * kGmLd + k] = (rr < m && k < ncb) ? __ldg(Y + rr * n + cb + k) : 0.f;
+    for (int u = 0; u < kU; ++u) {
+      const int r = tid / kGdK + u * (256 / kGdK);
+      const int64_t c = c0 + tid % kGdK;
+      va[u] = (c < c_end && i0 + r < m) ? __ldg(Y + (i0 + r) * n + c) : 0.f;
+      vb[u] = (c < c_end && j0 + r < m) ? __ldg(Y + (j0 + r) * n + c) : 0.f;
     }
-#pragma unroll 8
-    for (int q = tid; q < kGmN * kGmCols; q += 128) {
-      const int r = q / kGmCols, k = q % kGmCols;
-      const int64_t rj = j0 + r;
-      sYb[r * kGmLd + k] = (rj < m && k < ncb) ? __ldg(Y + rj * n + cb + k) : 0.f;
+  };
+  double sum[4] = {0.0, 0.0, 0.0, 0.0};
+  load(c_begin);
+  for (int64_t c0 = c_begin; c0 < c_end; c0 += kGdK) {
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int r = tid / kGdK + u * (256 / kGdK);  // a warp holds a row
+      auto scaled = [](float v, int *e) {
+        *e = above_exp_f32(__reduce_max_sync(0xffffffffu, __float_as_uint(v) & 0x7fffffffu));
+        const int h = *e / 2;
+        return v * __int_as_float((127 - h) << 23) * __int_as_float((127 - (*e - h)) << 23);
+      };
+      int e0, e1;
+      sa[r][tid % kGdK] = scaled(va[u], &e0);
+      sb[r][tid % kGdK] = scaled(vb[u], &e1);
+      if (tid % kGdK == 0) ea[r] = e0, eb[r] = e1;
     }
     __syncthreads();
-    uint32_t abits = 0;
-    for (int k = 0; k < ncb; ++k) abits = max(abits, __float_as_uint(sYa[tid * kGmLd + k]) & 0x7fffffffu);
-    const int ea = above_exp_f32(abits);
-    const int ash = 8 - ea, ash1 = min(ash, 120);
-    const float asc1 = __int_as_float((127 + ash1) << 23), asc2 = __int_as_float((127 + ash - ash1) << 23);
-    if (tid < kGmN) {
-      uint32_t bbits = 0;
-      for (int k = 0; k < ncb; ++k) bbits = max(bbits, __float_as_uint(sYb[tid * kGmLd + k]) & 0x7fffffffu);
-      const int eb = above_exp_f32(bbits), bsh = 8 - eb, bsh1 = min(bsh, 120);
-      s_eb[tid] = eb;
-      s_bsc[0][tid] = __int_as_float((127 + bsh1) << 23);
-      s_bsc[1][tid] = __int_as_float((127 + bsh - bsh1) << 23);
-    }
-    __syncthreads();
-    for (int j = 0; j < nch && ok; ++j, ++jglob) {
-      const int b = jglob & 1;
-      if (issued[b] > phase[b]) {  // the products that last read this buffer
-        ok = tc_wait(sb[b], (uint32_t)(phase[b] & 1));
-        ++phase[b];
-      }
-      ok = __syncthreads_and(ok ? 1 : 0) != 0;
-      if (!ok) break;
-      __nv_bfloat16 *a = sA + (size_t)b * kTcSlices * kASlice;
-      __nv_bfloat16 *bb = sB + (size_t)b * kTcSlices * kBSlice;
-#pragma unroll 4
-      for (int k = 0; k < kTcK; ++k) slices_f32(sYa[tid * kGmLd + j * kTcK + k], asc1, asc2, a + kmaj16(tid, k), kASlice);
-      for (int q = tid; q < kGmN * kTcK; q += 128) {
-        const int r = q / kTcK, k = q % kTcK;
-        slices_f32(sYb[r * kGmLd + j * kTcK + k], s_bsc[0][r], s_bsc[1][r], bb + kmaj16(r, k), kBSlice);
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (tid == 0) {
-        const uint32_t aB = aS + (uint32_t)(b * kTcSlices * kASlice * 2), bB = bS + (uint32_t)(b * kTcSlices * kBSlice * 2);
+    load(c0 + kGdK);
+    DF acc[2][2];
+#pragma unroll 2
+    for (int q = 0; q < kGdK; q += 4) {
+      float x[2][4], y[2][4];
 #pragma unroll
-        for (int L = 0; L < kTcLevels; ++L) {
-          const int s0 = L < kTcSlices ? 0 : L - (kTcSlices - 1);
-          const int s1 = L < kTcSlices ? L : kTcSlices - 1;
-          for (int sa = s0; sa <= s1; ++sa) {
-            const uint64_t ad = umma_desc(aB + (uint32_t)(sa * kASlice * 2), lbo, sbo);
-            const uint64_t bd = umma_desc(bB + (uint32_t)((L - sa) * kBSlice * 2), lbo, sbo);
-            const uint32_t acc = (j > 0 || sa != s0) ? 1u : 0u;  // a fresh accumulation per block
-            asm volatile(
-                "{ .reg .pred p; setp.ne.u32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(
-                    tmem + (uint32_t)(L * kGmN)),
-                "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                : "memory");
-          }
+      for (int h = 0; h < 2; ++h) {
+        *reinterpret_cast<float4 *>(x[h]) = *reinterpret_cast<const float4 *>(&sa[ia + 16 * h][q]);
+        *reinterpret_cast<float4 *>(y[h]) = *reinterpret_cast<const float4 *>(&sb[jb + 16 * h][q]);
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        DF &s = acc[t >> 1][t & 1];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const float a = x[t >> 1][z], b = y[t & 1][z], p = a * b, e = fmaf(a, b, -p);
+          const float w = s.hi + p, bp = w - s.hi;
+          s.lo += ((s.hi - (w - bp)) + (p - bp)) + e;
+          s.hi = w;
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sb[b])
-                     : "memory");
-      }
-      ++issued[b];
-    }
-    // this block's products complete (both buffers), then its levels into FP64
-    for (int b = 0; b < 2 && ok; ++b)
-      while (issued[b] > phase[b] && ok) {
-        ok = tc_wait(sb[b], (uint32_t)(phase[b] & 1));
-        ++phase[b];
-      }
-    ok = __syncthreads_and(ok ? 1 : 0) != 0;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!ok) break;
-#pragma unroll
-    for (int n0 = 0; n0 < kGmN; n0 += 16) {  // 16 columns of j at a time: five levels, then FP64
-      long long accx[16];
-#pragma unroll
-      for (int q = 0; q < 16; ++q) accx[q] = 0;
-#pragma unroll
-      for (int L = 0; L < kTcLevels; ++L) {
-        uint32_t v[16];
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(L * kGmN + n0);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-            : "r"(taddr));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-          accx[q] += (long long)__float2int_rn(__uint_as_float(v[q])) << (8 * (kTcLevels - 1 - L));
-      }
-#pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const int sh = ea + s_eb[n0 + q] - 16 - 8 * (kTcLevels - 1);
-        const int sh1 = min(max(sh, -1000), 1000);
-        accd[n0 + q] += ((double)accx[q] * pow2d(sh1)) * pow2d(sh - sh1);
+        const float w = s.hi + s.lo;
+        s.lo -= w - s.hi;
+        s.hi = w;
       }
     }
-    // every warp has read the levels (and s_eb) before the next block overwrites them
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int e = ea[ia + 16 * (t >> 1)] + eb[jb + 16 * (t & 1)];
+      auto shifted = [&](float f) {  // f 2^e
+        return f == 0.f ? 0.0 : __longlong_as_double(__double_as_longlong(f2d_exact(f)) + ((long long)e << 52));
+      };
+      sum[t] += shifted(acc[t >> 1][t & 1].hi);
+      sum[t] += shifted(acc[t >> 1][t & 1].lo);
+    }
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   }
-  if (!ok && tid == 0) {  // give products still in flight (bounded) time to end, then record
-    for (int b = 0; b < 2; ++b)
-      while (issued[b] > phase[b]) {
-        tc_wait(sb[b], (uint32_t)(phase[b] & 1));
-        ++phase[b];
-      }
-    atomicOr(err, kErrTimeout);
-    s_ok = 0;
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (ri < m)
+  double *dst = out + (size_t)blockIdx.y * m * m;
 #pragma unroll
-    for (int q = 0; q < kGmN; ++q)
-      if (j0 + q < m)
-        part[(int64_t)blockIdx.z * m * m + ri * m + j0 + q] = s_ok ? accd[q] : __longlong_as_double(0x7ff8000000000000ll);
-  __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+  for (int t = 0; t < 4; ++t) {
+    const int i = i0 + ia + 16 * (t >> 1), j = j0 + jb + 16 * (t & 1);
+    if (j <= i && i < m) dst[(int64_t)i * m + j] = dst[(int64_t)j * m + i] = sum[t];
+  }
 }
 
-// S[q] = the column ranges' partials added in order
 __global__ void gram_reduce_kernel(const double *part, int nr, int64_t mm, double *S) {
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < mm; q += (int64_t)gridDim.x * blockDim.x) {
     double t = 0.0;
@@ -621,26 +511,23 @@ size_t gram_part_elems(int64_t m) {
 }
 
 void launch_gram(Ctx *c, const float *Y, int64_t m, int64_t n, double *S, cudaStream_t s) {
-  if (!core_on_tensor_cores() || !c->gram_part || m > kGramMaxRows || m < 1 || n < 1) {
+  if (!core_on_tensor_cores() || m < 1 || n < 1 || m > (1 << 20)) {  // TUCKER_CORE_TC=0: FP64
     gram_f32(Y, m, n, S, s);
     return;
   }
-  const int64_t ti = (m + kGmM - 1) / kGmM, tj = (m + kGmN - 1) / kGmN;
-  // column ranges: enough CTAs to reach about 2 x SMs, at most kGramMaxRanges, at least 32 columns each
-  int64_t nr = std::max<int64_t>(1, std::min<int64_t>((2 * (int64_t)c->num_sms) / (ti * tj), kGramMaxRanges));
-  nr = std::min<int64_t>(nr, std::max<int64_t>(1, n / 32));
-  const int64_t cpr = (n + nr - 1) / nr;
+  const int64_t t = (m + kGdT - 1) / kGdT, tiles = t * (t + 1) / 2;
+  int64_t nr = 1;  // column ranges: about four blocks an SM
+  if (c->gram_part && m <= kGramMaxRows)
+    nr = std::max<int64_t>(1, std::min<int64_t>(4 * (int64_t)c->num_sms / tiles, kGramMaxRanges));
+  const int64_t cpr = ((n + nr - 1) / nr + kGdK - 1) / kGdK * kGdK;
   nr = (n + cpr - 1) / cpr;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  cudaStreamIsCapturing(s, &cap);
-  if (cap == cudaStreamCaptureStatusNone)
-    cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gm_smem_bytes());
-  gram_tc_kernel<<<dim3((unsigned)ti, (unsigned)tj, (unsigned)nr), 128, gm_smem_bytes(), s>>>(Y, m, n, cpr,
-                                                                                           c->gram_part, c->d_err);
+  gram_df_kernel<<<dim3((unsigned)tiles, (unsigned)nr), 256, 0, s>>>(Y, (int)m, n, cpr, nr > 1 ? c->gram_part : S);
   ::tk::count_launch();
-  const int64_t mm = m * m;
-  gram_reduce_kernel<<<(unsigned)std::min<int64_t>((mm + 255) / 256, 4096), 256, 0, s>>>(c->gram_part, (int)nr, mm, S);
-  ::tk::count_launch();
+  if (nr > 1) {
+    const int64_t mm = m * m;
+    gram_reduce_kernel<<<(unsigned)std::min<int64_t>((mm + 255) / 256, 4096), 256, 0, s>>>(c->gram_part, (int)nr, mm, S);
+    ::tk::count_launch();
+  }
 }
 
 // The core runs on the tensor cores (core_tc_kernel + core_reduce_kernel) where R <= 64 and
