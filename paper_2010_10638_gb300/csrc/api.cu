@@ -217,8 +217,12 @@ static tucker_status init_impl(Ctx *c, const uint32_t *coords, const float *vals
     c->sq_elems = rows;
   }
   for (int n = 0; n < N; ++n)
-    if (qrp_n_cols(c, n) == c->mode[n].P)
-      c->qgram_bytes = std::max(c->qgram_bytes, qrp_gram_bytes(c->mode[n].I, c->mode[n].P, c->ranks[n], c->num_sms));
+  {
+    const int64_t I = c->mode[n].I, P = c->mode[n].P;
+    const bool fat = qrp_n_cols(c, n) == I && P > I;
+    c->qgram_bytes = std::max(c->qgram_bytes, fat ? qrp_gram_bytes64(I, I, c->ranks[n], c->num_sms)
+                                                  : qrp_gram_bytes(I, P, c->ranks[n], c->num_sms));
+  }
   if (c->qgram_bytes && dev_alloc(c, &c->qgram, c->qgram_bytes) != cudaSuccess) {  // not needed: the cluster form
     cudaGetLastError();
     c->qgram = nullptr;
@@ -311,13 +315,13 @@ static tucker_status hooi_impl(Ctx *c, double *fit_out, cudaStream_t s) {
     QrpWork w;
     qrp_bind_work(&w, c->qw.V, mc.I, ncols, k, c->num_sms);
     w.err_out = c->d_err;  // a timed-out wait is reported by the next synchronising call
+    w.gram_ws = c->qgram;
+    w.gram_bytes = c->qgram_bytes;
     if (gram) {
       launch_gram(c, c->Y, mc.I, mc.P, c->gram, s);
       st = qrp_run_f64(c->gram, mc.I, mc.I, mc.I, k, c->U64[n], k, nullptr, nullptr, &w, c->num_sms, s);
     } else {
       if (norms) w.colsq = c->colsq;
-      w.gram_ws = c->qgram;
-      w.gram_bytes = c->qgram_bytes;
       st = qrp_run_f32(c->Y, mc.I, mc.P, mc.P, k, c->U64[n], k, nullptr, nullptr, &w, c->num_sms, s);
     }
     if (st != TUCKER_OK) return st;

@@ -89,7 +89,7 @@ struct QrpWork {
   // [n] column sums of squares of A given by the caller (FP32 A), or nullptr: the cluster
   // form then skips its own first pass over A and takes these as the initial norms
   const double *colsq = nullptr;
-  // FP32 A: workspace of the Gram form (qrp_gram.cu), or nullptr: not tried
+  // workspace of the Gram forms (qrp_gram.cu, qrp_gram64.cu), or nullptr: not tried
   void *gram_ws = nullptr;
   size_t gram_bytes = 0;
   // the cluster form runs only if this device word is not zero (nullptr: always)
@@ -128,7 +128,7 @@ struct Ctx {
   uint32_t *fib_iota = nullptr;  // fiber form: 0, 1, ..., F-1 (max F)
   float *fib_ones = nullptr;   // fiber form: 1.0f (max F)
   double *gram = nullptr;      // Y Y^T for fat unfoldings
-  double *gram_part = nullptr; // column-range partials of the tensor-core Gram matrix
+  double *gram_part = nullptr; // column-range partials of the Gram matrix
   float2 *sq_part = nullptr;   // column sums of squares of Y_(n): [rows][P_n] double-float pairs,
                                // one row per pipelined TTMc block, then one per split slice
   int64_t sq_elems = 0;        // pairs in sq_part (with the reduction's chunk sums after the rows)
@@ -322,17 +322,22 @@ void qrp_bind_work(QrpWork *w, void *base, int64_t m, int64_t n, int k, int nb);
 template <typename AT>
 bool qrp_cluster(const AT *A, int64_t m, int64_t n, int64_t lda, int k, double *Q, int64_t ldq, int64_t *piv,
                  double *rdiag, QrpWork *w, cudaStream_t s, cudaError_t *err);
-// Gram form (qrp_gram.cu): launches it and returns the device word that is not zero when it gave up
+// Gram form of tall FP32 matrices (qrp_gram.cu): launches it and returns the device word that is not zero when it gave up
 const uint32_t *qrp_gram(const float *A, int64_t m, int64_t n, int64_t lda, int k, double *Q, int64_t ldq, QrpWork *w,
                          int num_sms, cudaStream_t s, cudaError_t *err);
-bool qrp_gram_takes(int64_t m, int64_t n, int k, const QrpWork *w, int num_sms);  // the shape, with w's workspace
+bool qrp_gram_takes(const float *, int64_t m, int64_t n, int k, const QrpWork *w, int num_sms);  // shape, workspace
 size_t qrp_gram_bytes(int64_t m, int64_t n, int k, int num_sms);  // its workspace (0: not for this shape)
+// the same for small square FP64 matrices (qrp_gram64.cu)
+const uint32_t *qrp_gram(const double *A, int64_t m, int64_t n, int64_t lda, int k, double *Q, int64_t ldq, QrpWork *w,
+                         int num_sms, cudaStream_t s, cudaError_t *err);
+bool qrp_gram_takes(const double *, int64_t m, int64_t n, int k, const QrpWork *w, int num_sms);
+size_t qrp_gram_bytes64(int64_t m, int64_t n, int k, int num_sms);
 tucker_status qrp_run_f64(const double *A, int64_t m, int64_t n, int64_t lda, int k, double *Q, int64_t ldq,
                           int64_t *piv, double *rdiag, QrpWork *w, int nb, cudaStream_t s);
 tucker_status qrp_run_f32(const float *A, int64_t m, int64_t n, int64_t lda, int k, double *Q, int64_t ldq,
                           int64_t *piv, double *rdiag, QrpWork *w, int nb, cudaStream_t s);
 void gram_f32(const float *Y, int64_t m, int64_t n, double *S, cudaStream_t s);
-// S = Y Y^T on the tensor cores where it fits (m <= 1024, c->gram_part allocated), else gram_f32
+// S = Y Y^T in double-float (core.cu), with TUCKER_CORE_TC=0 in FP64 (gram_f32)
 void launch_gram(Ctx *c, const float *Y, int64_t m, int64_t n, double *S, cudaStream_t s);
 size_t gram_part_elems(int64_t m);  // partial buffer of launch_gram for an m x m Gram matrix (0: none)
 int qrp_blocks(int num_sms, int64_t m);

@@ -1118,21 +1118,19 @@ static tucker_status qrp_run(const AT *A, int64_t m, int64_t n, int64_t lda, int
   const char *form = std::getenv("TUCKER_QRP_FORM");
   if (!(form && std::strcmp(form, "multi") == 0)) {
     cudaError_t e = cudaSuccess;
-    if constexpr (sizeof(AT) == 4) {
-      // FP32, no pivots or diagonal asked for: from the Gram matrix; the cluster form runs behind
-      // it where it gave up (one that is asked for by name runs alone)
-      if (!form && !piv && !rdiag && qrp_gram_takes(m, n, k, w, nb)) {
-        w->plan_only = true;
-        const bool can = qrp_cluster<AT>(A, m, n, lda, k, Q, ldq, piv, rdiag, w, s, &e);
-        w->plan_only = false;
-        if (can) {
-          w->only_if = qrp_gram(A, m, n, lda, k, Q, ldq, w, nb, s, &e);
-          const bool behind = e == cudaSuccess && qrp_cluster<AT>(A, m, n, lda, k, Q, ldq, piv, rdiag, w, s, &e);
-          w->only_if = nullptr;
-          if (e != cudaSuccess) return TUCKER_ECUDA;
-          if (behind) return TUCKER_OK;
-          // (it could not be launched after all: the forms below write Q again in any case)
-        }
+    // no pivots or diagonal asked for: from the Gram matrix; the cluster form runs behind it
+    // where it gave up (one that is asked for by name runs alone)
+    if (!form && !piv && !rdiag && qrp_gram_takes(A, m, n, k, w, nb)) {
+      w->plan_only = true;
+      const bool can = qrp_cluster<AT>(A, m, n, lda, k, Q, ldq, piv, rdiag, w, s, &e);
+      w->plan_only = false;
+      if (can) {
+        w->only_if = qrp_gram(A, m, n, lda, k, Q, ldq, w, nb, s, &e);
+        const bool behind = e == cudaSuccess && qrp_cluster<AT>(A, m, n, lda, k, Q, ldq, piv, rdiag, w, s, &e);
+        w->only_if = nullptr;
+        if (e != cudaSuccess) return TUCKER_ECUDA;
+        if (behind) return TUCKER_OK;
+        // (it could not be launched after all: the forms below write Q again in any case)
       }
     }
     if (qrp_cluster<AT>(A, m, n, lda, k, Q, ldq, piv, rdiag, w, s, &e))

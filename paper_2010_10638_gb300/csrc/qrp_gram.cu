@@ -33,8 +33,7 @@
 #include <algorithm>
 #include <climits>
 
-#include "dfloat.cuh"
-#include "internal.cuh"
+#include "qrp_gram.cuh"
 #include "tc.cuh"
 
 namespace tk {
@@ -47,8 +46,6 @@ constexpr int kGK = 16;              // rows per stage
 constexpr int kGStages = 3;
 constexpr int kGSlices = 4, kGLevels = 4;
 constexpr int kGT = 512, kGWarps = kGT / 32;  // slicing threads; one more warp issues the products
-constexpr int kMaxK = 16;            // reflectors
-constexpr int kMaxN = 512;           // columns (one thread each in the pivot kernel)
 constexpr uint32_t kGCols = 512;     // tensor-memory columns: kGLevels * kGM
 constexpr int kGSlice = kGM * kGK;   // BF16 elements per slice of an operand
 constexpr uint32_t kGOperand = kGSlices * kGSlice * 2, kGStage = 2 * kGOperand;  // bytes
@@ -56,13 +53,6 @@ constexpr uint32_t kGOperand = kGSlices * kGSlice * 2, kGStage = 2 * kGOperand; 
 // the stages, and the tile's sums (in registers they spill)
 __host__ __device__ constexpr size_t qg_smem_bytes() {
   return (size_t)kGStages * kGStage + sizeof(float2) * kGM * kGM + 128;
-}
-
-// s += p, its rounding error into the low part (TwoSum)
-__device__ __forceinline__ void df_add1(DF &s, float p) {
-  const float t = s.hi + p, bp = t - s.hi;
-  s.lo += (s.hi - (t - bp)) + (p - bp);
-  s.hi = t;
 }
 
 // Exponents: ex[block][c] = e with |A[r, c]| < 2^e for the 256 rows r of the block (-128:
@@ -403,14 +393,15 @@ __device__ __forceinline__ void qg_warp_max(uint32_t &kh, uint32_t &kl, uint32_t
 // Pivoted Cholesky of S, k steps, one thread per column (one block), in double-float.
 //   r_c = (S[p, c] - sum_l r_lp r_lc) / r_p,  d_c -= r_c^2,  and in FP32 the coefficients w of column c in the
 //   pivot columns so far (S_11 w = S_1c): w_j = r_c / r_p, w_l -= w_j w_l(p)
-// With an error of at most kEps |a_i| |a_j| in every entry of S, that of a remaining norm (a Schur
-// complement) is at most kEps (|a_c| + sum_l |w_l| |a_l|)^2 to first order.  The pivot has to
+// With an error of at most eps |a_i| |a_j| in every entry of S, that of a remaining norm (a Schur
+// complement) is at most eps (|a_c| + sum_l |w_l| |a_l|)^2 to first order.  The pivot has to
 // exceed every other norm by more than both errors, and its own error 64 times.  (kEps: the
 // slices round what is below 2^-9 of a column's largest entry in 256 rows, by 2^-33 of that entry
 // at most and in either direction: 2^-33 |a_i| |a_j| where all of a column but one entry is so
 // small, about 2^-38 for normal entries.)
 constexpr float kEps = 1.2e-10f;  // 2^-33
 __global__ void __launch_bounds__(kMaxN) qg_pivot_kernel(const float2 *__restrict__ S, int n, int k,
+                                                         float eps,
                                                          int *__restrict__ piv, float2 *__restrict__ M,
                                                          uint32_t *flag) {
   extern __shared__ float2 qg_r[];  // [k][n] rows of R
@@ -432,6 +423,8 @@ __global__ void __launch_bounds__(kMaxN) qg_pivot_kernel(const float2 *__restric
     d.hi = v.x;
     d.lo = v.y;
   }
+  // (a norm whose products leave FP32's normal range, or that is not a number, decides nothing)
+  if (!(d.hi < 0x1p100f) || (d.hi > 0.f && d.hi < 0x1p-96f)) uncertain = true;
   const float na = sqrtf(fmaxf(d.hi, 0.f));
   float w[kMaxK], wsum = na;  // wsum = |a_c| + sum |w_l| |a_l|
 #pragma unroll
@@ -453,13 +446,13 @@ __global__ void __launch_bounds__(kMaxN) qg_pivot_kernel(const float2 *__restric
       uncertain = true;
       break;
     }
-    DF t;
+    DF t, row;  // (the row of S arrives while the products of the earlier rows are taken off)
     if (mine) {
       const float2 v = __ldcg(S + (size_t)p * n + c);
-      t.hi = v.x;
-      t.lo = v.y;
+      row.hi = v.x;
+      row.lo = v.y;
     }
-    const float e = kEps * wsum * wsum;
+    const float e = eps * wsum * wsum;
     if (c == p) {
       const DF inv = df_rsqrt(d);
       s_inv = make_float2(inv.hi, inv.lo);
@@ -476,6 +469,7 @@ __global__ void __launch_bounds__(kMaxN) qg_pivot_kernel(const float2 *__restric
     if (mine) {
 #pragma unroll 4
       for (int l = 0; l < j; ++l) df_sub_prod(t, qg_r[l * n + p], qg_r[l * n + c]);
+      df_add(t, row);
     }
     __syncthreads();
     DF inv, dp;
@@ -485,10 +479,7 @@ __global__ void __launch_bounds__(kMaxN) qg_pivot_kernel(const float2 *__restric
     dp.lo = s_dp.y;
     if (!done) uncertain = uncertain || !((dp.hi - d.hi) + (dp.lo - d.lo) > e + s_pe);
     if (mine) {
-      DF th;  // (t normalised)
-      th.hi = t.hi + t.lo;
-      th.lo = t.lo - (th.hi - t.hi);
-      const DF r = df_mul(th, inv);
+      const DF r = df_mul(t, inv);
       qg_r[j * n + c] = make_float2(r.hi, r.lo);
       df_sub_prod(d, make_float2(r.hi, r.lo), make_float2(r.hi, r.lo));
       const float dn = d.hi + d.lo;
@@ -721,25 +712,8 @@ __global__ void __launch_bounds__(kOT) qg_ortho_kernel(const float *__restrict__
     T64[i][l] = (double)v.hi + (double)v.lo;
   }
   __syncthreads();
-  bool close = false;
-  for (int j = 0; j < k; ++j) {  // elimination of the top block, a thread per entry
-    const float w = T[j][j], sg = w < 0.f ? -1.f : 1.f;
-    close = close || fabsf(w) < 2e-5f;
-    const float upd = (in && i > j && l > j) ? T[i][j] * (T[j][l] / (w + sg)) : 0.f;
-    __syncthreads();
-    if (in && i > j && l > j) T[i][l] -= upd;
-    if (tid == 0) sgn[j] = -sg;
-    __syncthreads();
-  }
-  if (close)  // (uniform: T is shared) a sign within FP32's error: again in FP64
-    for (int j = 0; j < k; ++j) {
-      const double w = T64[j][j], sg = w < 0.0 ? -1.0 : 1.0;
-      const double upd = (in && i > j && l > j) ? T64[i][j] * (T64[j][l] / (w + sg)) : 0.0;
-      __syncthreads();
-      if (in && i > j && l > j) T64[i][l] -= upd;
-      if (tid == 0) sgn[j] = -(float)sg;
-      __syncthreads();
-    }
+  // (a sign within FP32's error: again in FP64)
+  if (qg_signs(T, k, i, l, in, sgn)) qg_signs(T64, k, i, l, in, sgn);
   if (in) Wout[i * k + l] = i <= l ? make_float2(W[i][l].x * sgn[l], W[i][l].y * sgn[l]) : make_float2(0.f, 0.f);
 }
 
@@ -815,12 +789,32 @@ bool plan(int64_t m, int64_t n, int k, int num_sms, Plan *p) {
 
 }  // namespace
 
+void qg_reduce(const float2 *part, int ranges, int64_t n, float2 *S, cudaStream_t s) {
+  qg_reduce_kernel<<<(unsigned)std::min<int64_t>((n * n + 127) / 128, 2048), 128, 0, s>>>(part, ranges, n, S);
+  count_launch();
+}
+
+cudaError_t qg_pivots(const float2 *S, int64_t n, int k, float eps, int *piv, float2 *M, uint32_t *flag,
+                      cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(s, &cap);  // the attribute is set by the eager launches before any capture
+  if (cap == cudaStreamCaptureStatusNone) {
+    const cudaError_t e = cudaFuncSetAttribute(qg_pivot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)(sizeof(float2) * kMaxK * kMaxN));
+    if (e != cudaSuccess) return e;
+  }
+  const int threads = std::max(kMaxK * kMaxK, (int)((n + 31) / 32 * 32));
+  qg_pivot_kernel<<<1, threads, sizeof(float2) * (size_t)k * n, s>>>(S, (int)n, k, eps, piv, M, flag);
+  count_launch();
+  return cudaSuccess;
+}
+
 size_t qrp_gram_bytes(int64_t m, int64_t n, int k, int num_sms) {
   Plan p;
   return plan(m, n, k, num_sms, &p) ? p.total : 0;
 }
 
-bool qrp_gram_takes(int64_t m, int64_t n, int k, const QrpWork *w, int num_sms) {
+bool qrp_gram_takes(const float *, int64_t m, int64_t n, int k, const QrpWork *w, int num_sms) {
   Plan p;
   return w->gram_ws && plan(m, n, k, num_sms, &p) && p.total <= w->gram_bytes;
 }
@@ -838,15 +832,10 @@ const uint32_t *qrp_gram(const float *A, int64_t m, int64_t n, int64_t lda, int 
   float2 *W = reinterpret_cast<float2 *>(ws + p.W), *opart = reinterpret_cast<float2 *>(ws + p.opart);
   int *piv = reinterpret_cast<int *>(ws + p.piv);
   float2 *Q1 = reinterpret_cast<float2 *>(ws + p.q1);
-  const int pt = std::max(kMaxK * kMaxK, (int)((n + 31) / 32 * 32));
-  const size_t psmem = sizeof(float2) * (size_t)k * n;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  cudaStreamIsCapturing(s, &cap);  // the attributes are set by the eager launches before any capture
+  cudaStreamIsCapturing(s, &cap);  // the attribute is set by the eager launches before any capture
   if (cap == cudaStreamCaptureStatusNone) {
     *err = cudaFuncSetAttribute(qg_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qg_smem_bytes());
-    if (*err == cudaSuccess)
-      *err = cudaFuncSetAttribute(qg_pivot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)(sizeof(float2) * kMaxK * kMaxN));
     if (*err != cudaSuccess) return words;
   }
   if ((*err = cudaMemsetAsync(words, 0, 8, s)) != cudaSuccess) return words;
@@ -855,10 +844,8 @@ const uint32_t *qrp_gram(const float *A, int64_t m, int64_t n, int64_t lda, int 
   qg_gram_kernel<<<dim3((unsigned)p.tiles, (unsigned)p.ranges), kGT + 32, qg_smem_bytes(), s>>>(
       A, m, n, lda, p.rows_per, ex, part, words, w->err_out);
   count_launch();
-  qg_reduce_kernel<<<(unsigned)std::min<int64_t>((n * n + 127) / 128, 2048), 128, 0, s>>>(part, p.ranges, n, S);
-  count_launch();
-  qg_pivot_kernel<<<1, pt, psmem, s>>>(S, (int)n, k, piv, M, words);
-  count_launch();
+  qg_reduce(part, p.ranges, n, S, s);
+  if ((*err = qg_pivots(S, n, k, kEps, piv, M, words, s)) != cudaSuccess) return words;
   qg_ortho_kernel<<<p.oblocks, kOT, 0, s>>>(A, m, lda, k, piv, M, Q1, opart, words + 1, W, words);
   count_launch();
   qg_q_kernel<<<(unsigned)std::min<int64_t>((m + 15) / 16, 8 * (int64_t)num_sms), 256, 0, s>>>(Q1, m, k, W, words, Q,

@@ -69,6 +69,53 @@ def test_q_matches_oracle(m, a, b, k):
     np.testing.assert_allclose(Q, oracle.qrp(A.astype(np.float64), k).Q, atol=1e-10)
 
 
+@pytest.mark.parametrize("m,a,b,k", [
+    (12, 3, 5, 6),  # the smallest, a single tile and block
+    (31, 6, 6, 7),
+    (33, 6, 8, 16),  # one past a tile and two blocks
+    (64, 9, 9, 8),
+    (200, 16, 16, 16),
+    (257, 17, 16, 13),
+    (512, 20, 26, 16),  # the largest
+])
+def test_fat_branch(m, a, b, k, monkeypatch):
+    """m < ab: the QR of S = A A^T in FP64 (qrp_gram64.cu), against the cluster form on the same S:
+    both are backward stable, so 2^-53 times the condition of S (below 1e4) times a few dozen."""
+    A = matrix(a * b, m, 5 * m + a).T.copy()
+    _, Q = first_factor(A, a, b, k)
+    monkeypatch.setenv("TUCKER_QRP_FORM", "cluster")
+    _, want = first_factor(A, a, b, k)
+    np.testing.assert_allclose(Q.T @ Q, np.eye(k), atol=1e-13)
+    np.testing.assert_allclose(Q, want, atol=1e-10)
+
+
+@pytest.mark.parametrize("name", ["copies", "rank-deficient", "tiny", "huge"])
+def test_fat_branch_undecided_runs_the_cluster_form(name, monkeypatch):
+    A = matrix(120, 60, 9).T.copy()
+    if name == "copies":
+        A[30:] = A[:30]
+    elif name == "rank-deficient":
+        rng = np.random.default_rng(6)
+        A = (rng.integers(-8, 9, (60, 5)) @ rng.integers(-8, 9, (5, 120))).astype(np.float32)
+    else:  # entries of S below 2^-60, above 2^60
+        A *= np.float32(2.0 ** (-34 if name == "tiny" else 28))
+    _, Q = first_factor(A, 10, 12, 8)
+    monkeypatch.setenv("TUCKER_QRP_FORM", "cluster")
+    _, want = first_factor(A, 10, 12, 8)
+    np.testing.assert_array_equal(Q, want)
+
+
+@pytest.mark.parametrize("power", [-60, 60])
+def test_fat_branch_magnitudes(power, monkeypatch):
+    """S of entries near the ends of FP32's range, where their products leave it: a power of two
+    changes nothing but S's exponents."""
+    A = matrix(120, 60, 9).T.copy()
+    _, Q = first_factor(A * np.float32(2.0**power), 10, 12, 8)
+    monkeypatch.setenv("TUCKER_QRP_FORM", "cluster")
+    _, want = first_factor(A, 10, 12, 8)
+    np.testing.assert_allclose(Q, want, atol=1e-10)
+
+
 def hard(name):
     rng = np.random.default_rng(5)
     A = matrix(600, 48, 3)
