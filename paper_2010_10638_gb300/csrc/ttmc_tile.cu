@@ -155,9 +155,11 @@ __global__ void __launch_bounds__(kQCols) tile_q_kernel(const TileParams p, cons
     const int i = f / p.Gw, j = f % p.Gw, a = i / TB, b = i % TB;
     if (j < p.G && a < p.cA && b < p.cB) {
       const int R1 = p.nother == 1 ? 1 : p.R[1], R0 = p.R[0];
-      const int r = j / p.nB % p.nA * (p.cA == 8 ? 4 : p.cA) + a + (a >= 4 ? p.jA : 0);
-      const int q = j % p.nB * (p.cB == 8 ? 4 : p.cB) + b + (b >= 4 ? p.jB : 0);
-      if (r < R1 && q < R0) col = ((int64_t)(j / p.nB / p.nA) * R1 + r) * R0 + q;
+      int ja, jb, lead;
+      tile_split(j, p.nA, p.nB, ja, jb, lead);
+      const int r = ja * (p.cA == 8 ? 4 : p.cA) + a + (a >= 4 ? p.jA : 0);
+      const int q = jb * (p.cB == 8 ? 4 : p.cB) + b + (b >= 4 ? p.jB : 0);
+      if (r < R1 && q < R0) col = ((int64_t)lead * R1 + r) * R0 + q;
     }
   }
   for (int r = 0; r < R; ++r) gs[r * kQCols + threadIdx.x] = col >= 0 ? __ldg(G + r * p.P + col) : 0.f;

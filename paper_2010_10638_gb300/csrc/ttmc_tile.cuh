@@ -14,7 +14,7 @@
 // With 512 columns (5M nonzeros, ranks 8^4, one mode 0.24 - 0.29 ms) the multiply-adds: FMA
 // pipe 47%, issue slots 62% busy.
 //
-// One warp owns one work unit (reorder.cu), in steps of 32 nonzeros.  The factor rows and
+// One warp owns one work unit (reorder.cu), in steps of 32 or 16 nonzeros.  The factor rows and
 // the values of step t + 1 are copied to shared memory by cp.async while step t is
 // computed: no registers hold them, and a warp waits on no gather it has just issued.  A
 // nonzero's rows lie side by side in one record, at a record stride chosen for the bank groups
@@ -236,16 +236,32 @@ __host__ __device__ constexpr int tile_record(int used, int G, int n0, int n1, i
   return best;
 }
 
+// Tile j of a row: chunk jb of slot 0, ja of slot 1, and the number of its leading ranks.  Of j's
+// low bits the first is jb's, the next ja's, then come jb's others and ja's: a 16-byte read of
+// shared memory takes two cycles where no four consecutive lanes read more than two places, and
+// four otherwise (measured: with jb's bits lowest and four chunks or more, four).
+__host__ __device__ __forceinline__ void tile_split(int j, int nA, int nB, int &ja, int &jb, int &lead) {
+  if (nB >= 4 && nA >= 2) {
+    jb = (j & 1) | (j / 4 % (nB / 2)) << 1;
+    ja = (j / 2 & 1) | (j / (2 * nB) % (nA / 2)) << 1;
+  } else {
+    jb = j % nB;
+    ja = j / nB % nA;
+  }
+  lead = j / nB / nA;
+}
+
 // floats between the lanes' tile rows (an odd number of 16-byte pieces), and of a warp's memory
 __host__ __device__ constexpr int tile_row_stride(int TB) { return TB <= 4 ? 4 : 12; }
-__host__ __device__ constexpr int tile_warp_floats(int RS, int TB) {
-  return 64 * (RS + 1) + 32 * tile_row_stride(TB) + 2 * 32 * TB;
+__host__ __device__ constexpr int tile_warp_floats(int RS, int TB, int KS) {
+  return 2 * KS * (RS + 1) + 32 * tile_row_stride(TB) + 2 * 32 * TB;
 }
 
 constexpr int tile_min_blocks(int tile) {  // blocks of 128 threads an SM is to hold (registers)
   return tile > 56 ? 3 : tile > 40 ? 4 : tile > 30 ? 5 : tile > 20 ? 6 : 8;
 }
 
+// KS: nonzeros of a step.
 // NO: remaining modes whose indices are held in registers (1, 2, 3, or 7 for 4 to 7).
 //
 // ADJ (adjoint.cu): the TTMc of the residuals e_z = <Q(i_n, :), kron rows of z> - x_z, which it
@@ -254,7 +270,7 @@ constexpr int tile_min_blocks(int tile) {  // blocks of 128 threads an SM is to 
 // ranks 10^3: 0.40 ms; one thread per nonzero forming e_z alone took 1.71 ms, and the TTMc
 // 0.30 ms after it).  A group's lanes add their parts of the inner product by shuffles (Gw a
 // power of two; all groups step together).
-template <int NO, int TA, int TB, bool ADJ>
+template <int NO, int TA, int TB, bool ADJ, int KS = 32>
 __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB * (ADJ ? 2 : 1)))
     ttmc_tile_kernel(const __grid_constant__ TileParams p) {
   static_assert(NO > 1 || TA == 1, "one remaining mode: tiles of one row");
@@ -265,8 +281,8 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB * (AD
   if (u >= p.n_units) return;
   const int RS = p.RS, nother = NO <= 3 ? NO : p.nother;
   const int Gw = p.Gw, NG = p.NG, nA = p.nA, nB = p.nB;
-  float *ring = reinterpret_cast<float *>(tile_smem) + (size_t)w * tile_warp_floats(RS, TB);  // two steps of 32 records
-  float *rows = ring + 64 * (RS + 1);                                                          // one tile row per lane
+  float *ring = reinterpret_cast<float *>(tile_smem) + (size_t)w * tile_warp_floats(RS, TB, KS);  // two steps
+  float *rows = ring + 2 * KS * (RS + 1);                                                          // one tile row per lane
   int2 *place = reinterpret_cast<int2 *>(rows + 32 * tile_row_stride(TB));  // entries of Gw * TB columns
   const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
 
@@ -274,15 +290,17 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB * (AD
   const int g = lane / Gw;
   int j = (int)blockIdx.y * 32 + lane % Gw;
   if (j >= p.G) j = 0;  // no tile of its own: computes one, and `place` holds no place for it
-  const int jb = j % nB, ja = j / nB % nA;
-  int lead = j / nB / nA;
+  int jb, ja, lead;
+  tile_split(j, nA, nB, ja, jb, lead);
   const int R1 = NO == 1 ? 1 : p.R[1], R0 = p.R[0];
   // where entry (row 0, column b) of tile j of this block's tiles goes in a row of Y, and the
   // tile's first rank of slot 1 (chunks of eight, or fours of them, start at rank 4 j; others at cA j)
   for (int o = lane; o < Gw * TB; o += 32) {
-    const int oj = (int)blockIdx.y * 32 + o / TB, b = o % TB, ob = oj % nB, oa = oj / nB % nA;
+    const int oj = (int)blockIdx.y * 32 + o / TB, b = o % TB;
+    int ob, oa, ol;
+    tile_split(oj, nA, nB, oa, ob, ol);
     const int c = ob * (p.cB == 8 ? 4 : p.cB) + b + (b >= 4 ? p.jB : 0);
-    place[o] = make_int2(oj / nB / nA * R1 * R0 + c,
+    place[o] = make_int2(ol * R1 * R0 + c,
                          oj < p.G && b < p.cB && c < R0 ? oa * (p.cA == 8 ? 4 : p.cA) : INT_MIN / 2);
   }
   const uint32_t aoff = NO == 1 ? 0u : (uint32_t)(p.off[1] + 4 * ja) * 4u, boff = (uint32_t)(p.off[0] + 4 * jb) * 4u;
@@ -301,19 +319,19 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB * (AD
 
   const uint32_t e0 = __ldg(p.unit_e0 + u);
   const uint32_t e_end = (u + 1 < p.n_units) ? __ldg(p.unit_e0 + u + 1) : p.Z;
-  const int ntiles = (int)((e_end - e0 + 31u) / 32u);
+  const int ntiles = (int)((e_end - e0 + (uint32_t)KS - 1u) / (uint32_t)KS);
 
   uint32_t id[NO], vs = 0u;  // indices of the step whose copies are issued next (lane = position)
   auto load_ids = [&](int t) {
-    const uint32_t e = e0 + 32u * (uint32_t)t + (uint32_t)lane;
-    const bool in = e < e_end;
+    const uint32_t e = e0 + (uint32_t)KS * (uint32_t)t + (uint32_t)lane;
+    const bool in = (KS == 32 || lane < KS) && e < e_end;
 #pragma unroll
     for (int m = 0; m < NO; ++m) id[m] = (m < nother && in) ? __ldg(p.idx[m] + e) : 0u;
     vs = !in ? 0xffffffffu : p.vsrc ? __ldg(p.vsrc + e) : e;
   };
   auto issue = [&](int t) {  // copies of step t: values and rows (positions past the unit: row 0, not read)
-    const uint32_t st = ring_s + (uint32_t)(t & 1) * 32u * (uint32_t)RS * 4u;
-    if (vs != 0xffffffffu) tile_cp4(ring_s + (uint32_t)(64 * RS + 32 * (t & 1) + lane) * 4u, p.val + vs);
+    const uint32_t st = ring_s + (uint32_t)(t & 1) * (uint32_t)KS * (uint32_t)RS * 4u;
+    if (vs != 0xffffffffu) tile_cp4(ring_s + (uint32_t)(2 * KS * RS + KS * (t & 1) + lane) * 4u, p.val + vs);
 #pragma unroll
     for (int m = 0; m < NO; ++m) {
       if (m >= nother) break;
@@ -321,8 +339,9 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB * (AD
       const float *U = p.U[m] + 4 * c;
       uint32_t dst = st + (uint32_t)(z0 * RS + p.off[m] + 4 * c) * 4u;
       const uint32_t step = (uint32_t)(dz * RS) * 4u;
+      const int rounds = KS == 32 ? 1 << lq : 1 << (lq - 1);  // (KS = 16: rows of two pieces and more)
 #pragma unroll 4
-      for (int i = 0; i < (1 << lq); ++i, dst += step) {
+      for (int i = 0; i < rounds; ++i, dst += step) {
         const uint32_t r = __shfl_sync(kAll, id[m], z0 + i * dz);
         tile_cp16(dst, U + ((size_t)r << (lq + 2)));
       }
@@ -342,8 +361,8 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB * (AD
   if (ntiles > 1) load_ids(1);
 
   for (int t = 0; t < ntiles; ++t) {
-    const uint32_t e = e0 + 32u * (uint32_t)t;
-    const int nt = (int)min(32u, e_end - e);
+    const uint32_t e = e0 + (uint32_t)KS * (uint32_t)t;
+    const int nt = (int)min((uint32_t)KS, e_end - e);
     // slices of this step: bit q of `starts` is set where position q >= 1 starts one
     const uint32_t q = bound - e;
     uint32_t starts = __reduce_or_sync(kAll, q < 32u ? (1u << q) : 0u);
@@ -361,8 +380,8 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB * (AD
     __syncwarp();
     uint32_t eo = e + (uint32_t)lane;
     if (ADJ && p.esrc && lane < nt) eo = __ldg(p.esrc + eo);
-    const uint32_t st = ring_s + (uint32_t)((t & 1) * 32 * RS) * 4u;
-    const uint32_t xs = ring_s + (uint32_t)(64 * RS + 32 * (t & 1)) * 4u;
+    const uint32_t st = ring_s + (uint32_t)((t & 1) * KS * RS) * 4u;
+    const uint32_t xs = ring_s + (uint32_t)(2 * KS * RS + KS * (t & 1)) * 4u;
     uint32_t segs = starts | 1u;
     uint32_t kseg = kb;
     while (segs) {
@@ -489,7 +508,17 @@ constexpr size_t kTileSmem = 227 * 1024;  // shared memory a block may have
 template <int NO, int TA, int TB, bool ADJ = false>
 static cudaError_t run_tile(TileParams &p, int num_sms, cudaStream_t s) {
   auto kern = ttmc_tile_kernel<NO, TA, TB, ADJ>;
-  const size_t per = (size_t)tile_warp_floats(p.RS, TB) * sizeof(float);
+  int KS = 32;
+  // Order 3: 16 where the records are so wide (21 KB a warp for two steps of 32 records of 64
+  // floats) that an SM holds two blocks at most.  1M nonzeros, three modes: ranks 29^3 491 -> 391 us,
+  // 7 x 30 x 30 337 -> 272; where three blocks fit it loses (600,011, 12 x 7 x 20: 111 -> 127).
+  if constexpr (NO == 2)
+    if (p.lq[0] > 0 && p.lq[1] > 0 &&
+        kTileSmem / (kTileWarps * sizeof(float) * (size_t)tile_warp_floats(p.RS, TB, 32) + 1024) < 3) {
+      KS = 16;
+      kern = ttmc_tile_kernel<NO, TA, TB, ADJ, 16>;
+    }
+  const size_t per = (size_t)tile_warp_floats(p.RS, TB, KS) * sizeof(float);
   const int most = (int)std::min<size_t>(kTileWarps, kTileSmem / per);
   if (most < 1) return cudaErrorInvalidConfiguration;
   // small tensors: one warp per block reaches every SM

@@ -147,3 +147,20 @@ def test_units_of_many_slices(rows):
     ctx = T.tucker_init(dims, torch.as_tensor(coords.astype(np.int32)).cuda(), torch.as_tensor(vals).cuda(), ranks,
                         [torch.as_tensor(u).cuda() for u in U])
     check(T, ctx, dims, ranks, coords, vals, f32_round(U))
+
+
+@pytest.mark.parametrize("ranks", [(8, 29, 29), (8, 31, 32), (7, 30, 64)])
+def test_steps_of_sixteen(ranks):
+    """Records of 64 floats and more are taken 16 at a time: slices that end on either side of a step,
+    and rows of four and eight chunks, whose tiles are numbered in another order."""
+    T = lib()
+    dims = (8, 90, 80)
+    rng = np.random.default_rng(zlib.crc32(repr(ranks).encode()))
+    i = np.repeat(np.arange(8), [1, 15, 16, 17, 31, 0, 33, 300])
+    jk = np.stack(np.unravel_index(rng.permutation(90 * 80)[:i.size], (90, 80)))
+    coords = np.concatenate([i[None], jk]).astype(np.uint32)
+    vals = rng.standard_normal(i.size).astype(np.float32)
+    U = [rng.standard_normal((d, r)) for d, r in zip(dims, ranks)]
+    ctx = T.tucker_init(dims, torch.as_tensor(coords.astype(np.int32)).cuda(), torch.as_tensor(vals).cuda(), ranks,
+                        [torch.as_tensor(u).cuda() for u in U])
+    check(T, ctx, dims, ranks, coords, vals, f32_round(U))
