@@ -6,7 +6,7 @@
 //   1. one histogram kernel counts the first pass's digits and optionally validates the
 //      input; every pass counts the next pass's digits while it moves the records (a digit's
 //      global count does not depend on the order of the records);
-//   2. one kernel per pass: each block claims the next tile of 8192 records and ranks them
+//   2. one kernel per pass: each block claims the next tile of 8192 (or 2048) records and ranks them
 //      by digit (peer lanes of equal digit found by one ballot per digit bit; stable),
 //      publishes its digit counts, finds the counts of all earlier tiles by a decoupled
 //      look-back over a per-tile status word, and writes every word of the tile out in
@@ -24,8 +24,12 @@ namespace tk {
 
 constexpr int kRxThreads = 512;
 constexpr int kRxWarps = kRxThreads / 32;
-constexpr int kRxSteps = 16;                         // 32-record steps per warp
-constexpr int kRxTile = kRxWarps * kRxSteps * 32;    // 8192 records per tile
+// A tile is kRxWarps warps of `Steps` steps of 32 records: 8192 records, or 2048 where tiles of
+// 8192 would leave most SMs without one (three sorts of an initialisation, with the rest of it:
+// 300,000 nonzeros 737 -> 689 us, 100,000 662 -> 636; 1M 773 -> 819, 10M 2,301 -> 2,557)
+constexpr int rx_tile(int Steps) { return kRxWarps * Steps * 32; }
+constexpr int64_t kRxSmall = 1 << 19;
+static int rx_steps(int64_t n) { return n <= kRxSmall ? 4 : 16; }
 constexpr int kRxBins = 256;                         // digits of at most 8 bits
 constexpr int kRxMaxPasses = 4 * kMaxOrder + 4;
 constexpr uint64_t kRxFlagAgg = 1ull << 32;          // status: this tile's own counts
@@ -147,21 +151,24 @@ __device__ __forceinline__ void rx_store(unsigned long long *p, unsigned long lo
   *reinterpret_cast<volatile unsigned long long *>(p) = v;
 }
 
+template <int Steps>
 struct RxSmem {
   uint32_t wcnt[kRxWarps][kRxBins];  // per-warp digit counts, then the warp's offset in the tile bucket
   uint32_t tstart[kRxBins];          // first local position of each digit
   uint32_t gbase[kRxBins];           // global position of that first record
-  uint32_t buf[kRxTile];             // one word of the tile, by local position
-  uint32_t gidx[kRxTile];            // local position -> global position
+  uint32_t buf[rx_tile(Steps)];             // one word of the tile, by local position
+  uint32_t gidx[rx_tile(Steps)];            // local position -> global position
   uint32_t nh[kRxBins];               // this tile's counts of the next pass's digits
   uint32_t wsum[kRxWarps];
   uint32_t tile;
   uint32_t bad;
 };
 
-__global__ void __launch_bounds__(kRxThreads, 2) rx_pass_kernel(RxPassArgs a) {
+template <int kRxSteps>
+__global__ void __launch_bounds__(kRxThreads, kRxSteps > 8 ? 2 : 4) rx_pass_kernel(RxPassArgs a) {
+  constexpr int kRxTile = rx_tile(kRxSteps);
   extern __shared__ __align__(16) unsigned char rx_raw[];
-  RxSmem &sm = *reinterpret_cast<RxSmem *>(rx_raw);
+  RxSmem<kRxSteps> &sm = *reinterpret_cast<RxSmem<kRxSteps> *>(rx_raw);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const uint32_t nbins = 1u << a.bits, mask = nbins - 1u;
   if (tid == 0) {
@@ -244,25 +251,28 @@ __global__ void __launch_bounds__(kRxThreads, 2) rx_pass_kernel(RxPassArgs a) {
   }
   __syncthreads();
 
-  // ---- look-back over earlier tiles (one thread per digit)
+  // ---- look-back over earlier tiles (one thread per digit), the words of eight tiles in flight
+  //      (one at a time the initialisation of 1M skewed nonzeros took 977 us instead of 930)
   if (tid < kRxBins && (uint32_t)tid < nbins && tile > 0) {
     uint32_t excl = 0;
-    bool ok = true;
-    for (int64_t t = (int64_t)tile - 1; t >= 0;) {
-      unsigned long long v = rx_load(a.status + t * kRxBins + tid);
-      uint32_t polls = 0;
-      while ((v >> 32) == 0ull) {
-        if (++polls >= a.spin) break;
-        if (polls > 64) __nanosleep(128);
-        v = rx_load(a.status + t * kRxBins + tid);
+    bool ok = true, done = false;
+    for (int64_t t = (int64_t)tile - 1; t >= 0 && ok && !done; t -= 8) {
+      unsigned long long v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = t >= u ? rx_load(a.status + (t - u) * kRxBins + tid) : kRxFlagPre;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (!ok || done) continue;
+        uint32_t polls = 0;
+        while ((v[u] >> 32) == 0ull) {
+          if (++polls >= a.spin) break;
+          if (polls > 64) __nanosleep(128);
+          v[u] = rx_load(a.status + (t - u) * kRxBins + tid);
+        }
+        ok = (v[u] >> 32) != 0ull;
+        if (ok) excl += (uint32_t)v[u];
+        done = (v[u] >> 32) == (kRxFlagPre >> 32);
       }
-      if ((v >> 32) == 0ull) {
-        ok = false;
-        break;
-      }
-      excl += (uint32_t)v;
-      if ((v >> 32) == (kRxFlagPre >> 32)) break;
-      --t;
     }
     rx_store(a.status + (int64_t)tile * kRxBins + tid, kRxFlagPre | (uint32_t)(excl + tot));
     if (!ok) {
@@ -362,7 +372,8 @@ size_t radix_scratch_bytes(int64_t n, int nwords, const RadixKey *keys, int nkey
   RxPass pass[kRxMaxPasses];
   const int np = rx_plan(keys, nkeys, pass);
   if (np < 0) return 0;
-  const int64_t tiles = std::max<int64_t>(rx_cdiv(n, kRxTile), 1);
+  // the tiles of n records or any fewer (a sort of what is left after duplicates were added up)
+  const int64_t tiles = std::max<int64_t>({rx_cdiv(n, rx_tile(16)), rx_cdiv(std::min(n, kRxSmall), rx_tile(4)), 1});
   size_t b = 0;
   b += sizeof(unsigned long long) * (size_t)(np * tiles * kRxBins);  // status
   b += sizeof(uint32_t) * (size_t)(np * kRxBins + np + 64);           // histograms + tile counters
@@ -386,7 +397,7 @@ int radix_sort_records(int64_t n, const RadixRecords &r, const RadixKey *keys, i
   for (int q = 0; q < nvalid; ++q)
     if (!r.in[q]) return -1;
   if (scratch_bytes < radix_scratch_bytes(n, r.nwords, keys, nkeys)) return -1;
-  const int64_t tiles = std::max<int64_t>(rx_cdiv(n, kRxTile), 1);
+  const int64_t tiles = std::max<int64_t>(rx_cdiv(n, rx_tile(rx_steps(n))), 1);
   uint8_t *p = rx_align(static_cast<uint8_t *>(scratch));
   auto *status = reinterpret_cast<unsigned long long *>(p);
   p = rx_align(p + sizeof(unsigned long long) * (size_t)(np * tiles * kRxBins));
@@ -444,9 +455,10 @@ int radix_sort_records(int64_t n, const RadixRecords &r, const RadixKey *keys, i
     }
     return cudaGetLastError() == cudaSuccess ? 0 : -2;
   }
-  if (cudaFuncSetAttribute(rx_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RxSmem)) !=
-      cudaSuccess)
-    return -2;
+  const bool small = rx_steps(n) == 4;
+  const auto kern = small ? rx_pass_kernel<4> : rx_pass_kernel<16>;
+  const size_t smem = small ? sizeof(RxSmem<4>) : sizeof(RxSmem<16>);
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -2;
   const uint32_t *cur[kRadixMaxWords];
   for (int q = 0; q < r.nwords; ++q) cur[q] = r.in[q];
   for (int k = 0; k < np; ++k) {
@@ -473,7 +485,7 @@ int radix_sort_records(int64_t n, const RadixRecords &r, const RadixKey *keys, i
     a.err = err;
     a.spin = kRxSpin;
     if (n > 0) {
-      rx_pass_kernel<<<(unsigned)tiles, kRxThreads, sizeof(RxSmem), s>>>(a);
+      kern<<<(unsigned)tiles, kRxThreads, smem, s>>>(a);
       ::tk::count_launch();
     }
     for (int q = 0; q < r.nwords; ++q) cur[q] = a.out[q];
@@ -490,7 +502,7 @@ __global__ void rx_iota_kernel(uint32_t *out, int64_t n) {
 // counter starts at 1): its look-back waits for counts that never come, gives up after
 // `polls` polls and stores nothing.  Returns the error word (kErrTimeout expected).
 int radix_selftest_wait(uint32_t polls, cudaStream_t s, uint32_t *err_out) {
-  const int64_t n = 2 * (int64_t)kRxTile;
+  const int64_t n = 2 * (int64_t)rx_tile(16);
   uint32_t *words = nullptr;  // in [n], out [n], hist [256], counter, error word
   unsigned long long *status = nullptr;
   if (cudaMallocAsync(reinterpret_cast<void **>(&words), sizeof(uint32_t) * (size_t)(2 * n + kRxBins + 2), s) !=
@@ -506,7 +518,7 @@ int radix_selftest_wait(uint32_t polls, cudaStream_t s, uint32_t *err_out) {
   if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(unsigned long long) * 2 * kRxBins, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ctr, &one, sizeof(uint32_t), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(rx_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RxSmem));
+    e = cudaFuncSetAttribute(rx_pass_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RxSmem<16>));
   if (e == cudaSuccess) {
     RxPassArgs a{};
     a.n = n;
@@ -521,7 +533,7 @@ int radix_selftest_wait(uint32_t polls, cudaStream_t s, uint32_t *err_out) {
     a.tile_ctr = ctr;
     a.err = err;
     a.spin = polls;
-    rx_pass_kernel<<<1, kRxThreads, sizeof(RxSmem), s>>>(a);
+    rx_pass_kernel<16><<<1, kRxThreads, sizeof(RxSmem<16>), s>>>(a);
     e = cudaGetLastError();
   }
   *err_out = 0;
@@ -535,7 +547,8 @@ int radix_selftest_wait(uint32_t polls, cudaStream_t s, uint32_t *err_out) {
 cudaError_t preload_radix_kernels() {
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, rx_hist_kernel);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, rx_pass_kernel);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, rx_pass_kernel<4>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, rx_pass_kernel<16>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, rx_iota_kernel);
   return e;
 }
