@@ -474,17 +474,17 @@ def run_mine(args):
     q_bytes = sum(qbytes) / len(qbytes)
     one_pass = sum(w.dims[n] * ctx.P(n) * 4.0 + 2.0 * w.dims[n] * w.ranks[n] * 8.0 for n in big) / len(big)
     k_q = w.ranks[big[0]]
-    qrp_roof = {"kernel": f"qrp_cluster_kernel<float> on the {max(w.dims)} x {ctx.P(big[0])} unfoldings",
+    qrp_roof = {"kernel": f"Gram-form QRP (qg_* kernels) of the {max(w.dims)} x {ctx.P(big[0])} unfoldings",
                 "bound": "latency",
                 "achieved": one_pass / (q_ms * 1e-3) / 1e9, "peak": hbm_peak, "unit": "GB/s",
                 "frac": one_pass / (q_ms * 1e-3) / 1e9 / hbm_peak,
                 "traffic": None,
                 "peak_source": hbm_src, "dram_bytes_per_launch": one_pass, "avg_launch_ms": q_ms,
                 "us_per_reflector": q_ms * 1e3 / k_q,
-                "note": "DRAM traffic is about one pass over the FP32 Y plus V and Q (the other k passes of the "
-                        "column sums read shared memory and L2); the step is bound by the k dependent reflector "
-                        "steps (one grid barrier, a cluster reduction and FP64 dependent chains each), not by a "
-                        "memory or arithmetic roof; traffic is not captured (the kernel is kept off ncu)"}
+                "note": "the FP32 Y is read twice (exponents, Gram matrix), Q_1 written and read, Q written; bound "
+                        "by the slicing of Y for the tensor cores and, after it, by the latency of k pivot steps "
+                        "in one block; bytes and rate here are those of one pass over Y, V and Q, as for the "
+                        "reflector-by-reflector form"}
     dominant = ttmc_roof if ttmc_total >= qrp_total else qrp_roof
 
     cpu = None
@@ -516,9 +516,10 @@ def run_mine(args):
             "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": w.name, "dims": list(w.dims), "nnz": w.nnz, "nnz_coalesced": Zc,
                        "ranks": list(w.ranks), "l2": "flushed between timed steps (256 MiB write)",
-                       "precision": "TTMc FP32 (FP32 products and sums); QRP: FP64 storage, norms, reflectors, R "
-                                    "and T, with A^T y summed in double-float FP32 pairs around a power-of-two "
-                                    "offset (about 2^-49 s1 per product) and Q formed as double-float sums; core "
+                       "precision": "TTMc FP32 (FP32 products and sums); QRP: pivots and R from Y^T Y (exact "
+                                    "8-bit slices on the tensor cores, double-float sums, 2^-33), Q from the "
+                                    "pivot columns in double-float with its orthogonality corrected (2e-14), "
+                                    "stored in FP64; core "
                                     "on the tensor cores: Y (FP32) and U_N (FP64) cut into four exact 8-bit "
                                     "fixed-point slices per column, BF16 products summed exactly (integer) in "
                                     "FP32 tensor memory, levels combined in 64-bit integers, row ranges and fit "
