@@ -749,16 +749,21 @@ struct Plan {
   int64_t blocks;
 };
 
-// Six reflectors and more.  It takes 50 to 60 us for the smallest matrices, the cluster form 8 us
-// a reflector there and 22 us:
+// Six reflectors and more, four and five where the matrix is tall and narrow; up to 64 columns a
+// reflector where it is tall and wide.  It takes 50 to 60 us for the smallest matrices and S grows
+// with m n^2; the cluster form takes 8 us a reflector for the smallest and 22 us at 50,000 x 256:
 //   m x n, k            here   cluster (us)        m x n, k             here   cluster
 //   200 x 64, 4           58        52             200 x 64, 6            60        67
 //   512 x 128, 4          59        53             512 x 128, 6           59        69
-//   20,000 x 64, 2        77        66             20,000 x 64, 6         81       113
+//   2,000 x 128, 4        63        67             6,000 x 256, 4         74        73
+//   10,000 x 64, 5        70       151             6,000 x 256, 5         75        84
+//   20,000 x 512, 5      174       138             4,000 x 512, 6         89       113
 //   100 x 64, 8           61        82             4,000 x 512, 16       112       248
 //   1,000 x 256, 16       83       186             50,000 x 256, 16      180       363
 bool plan(int64_t m, int64_t n, int k, int num_sms, Plan *p) {
-  if (k < 6 || k > kMaxK || n < k || n > kMaxN || m < n || m < 2 * k) return false;
+  if (k < 4 || k > kMaxK || n < k || n > kMaxN || m < n || m < 2 * k) return false;
+  if (k < 6 && (m < 2000 || n > 128 * (k - 3))) return false;
+  if (m > 4000 && n > 64 * k) return false;
   const int t = (int)((n + kGM - 1) / kGM);
   p->tiles = t * (t + 1) / 2;
   const int64_t blocks = (m + kGRows - 1) / kGRows;

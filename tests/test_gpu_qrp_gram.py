@@ -60,6 +60,8 @@ def matrix(m, n, seed):
     (2003, 11, 35, 13),
     (10_000, 8, 8, 8),  # ranges of rows that start in the middle of a block
     (38_917, 5, 6, 10),
+    (2000, 8, 16, 4),  # tall and narrow: four and five reflectors
+    (5731, 5, 25, 5),
 ])
 def test_q_matches_oracle(m, a, b, k):
     A = matrix(m, a * b, 7 * m + a)
