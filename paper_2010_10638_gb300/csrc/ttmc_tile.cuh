@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB * (AD
   acc.clear();
   TileAcc<TA, TB> qt;  // ADJ: this lane's tile of the slice's row of Q
   bool fresh = true;   //      not loaded yet
-  DF sq;
+  double sq = 0.0;  // in FP64: the squares of FP32 residuals leave FP32's range
   uint32_t kb = __ldg(p.unit_k0 + u);
   uint32_t bound = (kb + 1u + lane <= p.S) ? __ldg(p.sptr + kb + 1u + lane) : 0xffffffffu;
   load_ids(0);
@@ -489,17 +489,17 @@ __global__ void __launch_bounds__(kTileWarps * 32, tile_min_blocks(TA * TB * (AD
       if (lane < nt) {
         const float r = tile_lds1(xs + (uint32_t)lane * 4u);
         p.e_out[eo] = r;
-        df_fma(sq, r, r, 0.f);
+        const double rd = f2d_exact(r);
+        sq = fma(rd, rd, sq);
       }
       __syncwarp();  // read before the next step's values are copied there
     }
     kb = kb_next;
   }
   if constexpr (ADJ) {
-    double s = (double)sq.hi + (double)sq.lo;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kAll, s, o);
-    if (lane == 0) p.sq_part[u] = s;
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(kAll, sq, o);
+    if (lane == 0) p.sq_part[u] = sq;
   }
 }
 
