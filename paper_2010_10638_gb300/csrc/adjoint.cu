@@ -268,9 +268,11 @@ static cudaError_t launch_du(Ctx *c, int n, const float *G, int64_t PR, float *d
   for (int m = 0; m < c->N; ++m) uf.R[m] = c->ranks[m];
   const int nr = kDuThreads / R;
   const int64_t smem = ((int64_t)nr * (mc.P + 8) + mc.P * R) * (int64_t)sizeof(float);
-  if (smem <= 200 * 1024) {
+  constexpr int kDuSmem = 200 * 1024;
+  if (smem <= kDuSmem) {
     const size_t bytes = (size_t)(nr * du_stride((int)mc.P) + (int)mc.P * R) * sizeof(float);
-    const cudaError_t e = cudaFuncSetAttribute(adj_du_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    // (the most of any call: the attribute is the function's, shared by all contexts)
+    const cudaError_t e = cudaFuncSetAttribute(adj_du_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDuSmem);
     if (e != cudaSuccess) return e;
     const int64_t tiles = (mc.I + nr - 1) / nr;
     const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(4, (int64_t)(220 * 1024) / (int64_t)bytes));

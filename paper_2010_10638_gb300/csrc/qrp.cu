@@ -984,8 +984,10 @@ static bool qrp_persistent(const AT *A, int64_t m, int64_t n, int64_t lda, int k
   const size_t stage_bytes = std::max<size_t>((size_t)kPStage * 8, (size_t)k * k * sizeof(double));
   const size_t smem = perm_bytes + ((stage_bytes + 15) & ~(size_t)15) + (size_t)k * k * sizeof(double);
   auto kern = qrp_persistent_kernel<AT>;
-  // the 48 KB default bounds static + dynamic shared memory together: always opt in
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
+  // the 48 KB default bounds static + dynamic shared memory together: always opt in, to the most of
+  // any call (n = 8192, k = 64; the attribute is the function's, shared by all contexts)
+  constexpr size_t kMost = 8192 * sizeof(int) + std::max<size_t>(kPStage * 8, 64 * 64 * 8) + 64 * 64 * 8;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost) != cudaSuccess) return false;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPThreads, smem) != cudaSuccess || per_sm < 1)
     return false;

@@ -523,7 +523,9 @@ static cudaError_t run_tile(TileParams &p, int num_sms, cudaStream_t s) {
   if (most < 1) return cudaErrorInvalidConfiguration;
   // small tensors: one warp per block reaches every SM
   const int W = (int)std::max<int64_t>(1, std::min<int64_t>(most, p.n_units / num_sms));
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(per * W));
+  // the most a block may have, not this launch's: the attribute is the function's, and a call on
+  // another context may set it between here and the launch
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((p.n_units + W - 1) / W), (unsigned)((p.G + 31) / 32));
   kern<<<grid, 32 * W, per * W, s>>>(p);
