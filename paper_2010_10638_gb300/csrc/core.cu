@@ -482,8 +482,9 @@ __global__ void __launch_bounds__(256) gram_df_kernel(const float *__restrict__ 
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const int e = ea[ia + 16 * (t >> 1)] + eb[jb + 16 * (t & 1)];
-      auto shifted = [&](float f) {  // f 2^e
-        return f == 0.f ? 0.0 : __longlong_as_double(__double_as_longlong(f2d_exact(f)) + ((long long)e << 52));
+      auto shifted = [&](float f) {  // f 2^e (of an overflowed row: infinity or NaN as it is)
+        if (f == 0.f || !isfinite(f)) return (double)f;
+        return __longlong_as_double(__double_as_longlong(f2d_exact(f)) + ((long long)e << 52));
       };
       sum[t] += shifted(acc[t >> 1][t & 1].hi);
       sum[t] += shifted(acc[t >> 1][t & 1].lo);
