@@ -414,7 +414,8 @@ static bool core_on_tensor_cores();
 // slicing and hand-overs: 200 x 256 32 -> 11 us with the sum of the ranges; with the QRP that
 // follows 64 x 3,600 288 -> 191, 200 x 1,280 151 -> 104, 1,000 x 1,056 708 -> 652, 1,000 x 4,096
 // 1,682 -> 1,599.
-constexpr int kGramMaxRows = 1024;  // above, tiles alone fill the GPU: one range
+constexpr int kGramMaxRows = 1024;  // above, in FP64 (gram_f32): slower (1,100 x 2,048, with the QRP, 11.7 ms
+                                    // for 0.94), but its error is 2^-53 for 2^-46
 constexpr int kGramMaxRanges = 8;   // column ranges (partial sets)
 constexpr int kGdT = 32, kGdK = 32, kGdLd = kGdK + 4;
 __global__ void __launch_bounds__(256) gram_df_kernel(const float *__restrict__ Y, int m, int64_t n,
@@ -512,14 +513,13 @@ size_t gram_part_elems(int64_t m) {
 }
 
 void launch_gram(Ctx *c, const float *Y, int64_t m, int64_t n, double *S, cudaStream_t s) {
-  if (!core_on_tensor_cores() || m < 1 || n < 1 || m > (1 << 20)) {  // TUCKER_CORE_TC=0: FP64
+  if (!core_on_tensor_cores() || !c->gram_part || m > kGramMaxRows || m < 1 || n < 1) {  // TUCKER_CORE_TC=0: FP64
     gram_f32(Y, m, n, S, s);
     return;
   }
   const int64_t t = (m + kGdT - 1) / kGdT, tiles = t * (t + 1) / 2;
-  int64_t nr = 1;  // column ranges: about four blocks an SM
-  if (c->gram_part && m <= kGramMaxRows)
-    nr = std::max<int64_t>(1, std::min<int64_t>(4 * (int64_t)c->num_sms / tiles, kGramMaxRanges));
+  // column ranges: about four blocks an SM
+  int64_t nr = std::max<int64_t>(1, std::min<int64_t>(4 * (int64_t)c->num_sms / tiles, kGramMaxRanges));
   const int64_t cpr = ((n + nr - 1) / nr + kGdK - 1) / kGdK * kGdK;
   nr = (n + cpr - 1) / cpr;
   gram_df_kernel<<<dim3((unsigned)tiles, (unsigned)nr), 256, 0, s>>>(Y, (int)m, n, cpr, nr > 1 ? c->gram_part : S);

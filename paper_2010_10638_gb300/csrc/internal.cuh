@@ -337,7 +337,7 @@ tucker_status qrp_run_f64(const double *A, int64_t m, int64_t n, int64_t lda, in
 tucker_status qrp_run_f32(const float *A, int64_t m, int64_t n, int64_t lda, int k, double *Q, int64_t ldq,
                           int64_t *piv, double *rdiag, QrpWork *w, int nb, cudaStream_t s);
 void gram_f32(const float *Y, int64_t m, int64_t n, double *S, cudaStream_t s);
-// S = Y Y^T in double-float (core.cu), with TUCKER_CORE_TC=0 in FP64 (gram_f32)
+// S = Y Y^T in double-float up to 1,024 rows (core.cu), above and with TUCKER_CORE_TC=0 in FP64 (gram_f32)
 void launch_gram(Ctx *c, const float *Y, int64_t m, int64_t n, double *S, cudaStream_t s);
 size_t gram_part_elems(int64_t m);  // partial buffer of launch_gram for an m x m Gram matrix (0: none)
 int qrp_blocks(int num_sms, int64_t m);

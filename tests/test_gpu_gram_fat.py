@@ -44,3 +44,13 @@ def test_overflowed_row_stays_visible(m, a, b, row, what):
     assert (np.isinf(Y[row]) if what == "inf" else np.isnan(Y[row])).all()
     assert np.isfinite(np.delete(Y, row, 0)).all()
     assert not np.isfinite(Q).all()
+
+
+@pytest.mark.parametrize("m,a,b", [(1025, 33, 34), (1100, 33, 34)])
+def test_above_1024_rows_in_fp64(m, a, b, monkeypatch):
+    """More than 1,024 rows: S in FP64, as with TUCKER_CORE_TC=0, bit for bit."""
+    A = fat(m, a * b, m)
+    _, Q = first_factor(A, a, b, 8)
+    monkeypatch.setenv("TUCKER_CORE_TC", "0")
+    _, want = first_factor(A, a, b, 8)
+    np.testing.assert_array_equal(Q, want)
