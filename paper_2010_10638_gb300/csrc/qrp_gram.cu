@@ -5,8 +5,8 @@
 // are those of a Cholesky factorisation with the same pivot rule.  So A is read once for
 // S = A^T A, on the tensor cores, instead of once per reflector; the chain of k pivot steps
 // runs in one block on n numbers; and Q follows from the k pivot columns alone:
-//   1  qg_exp_kernel, qg_gram_kernel  S, exact fixed-point slices as in core.cu (error below
-//                        2^-33 of |a_i| |a_j|), ranges of rows in double-float pairs
+//   1  qg_exp_kernel, qg_gram_kernel  S, fixed-point slices as in core.cu (error: see qg_eps;
+//                        usually 2^-38 of |a_i| |a_j|), ranges of rows in double-float pairs
 //   2  qg_reduce_kernel  the ranges added in order
 //   3  qg_pivot_kernel   pivots p_1 .. p_k, the triangle R_1, its inverse (double-float)
 //   4  qg_ortho_kernel   E = Q_1^T Q_1 - I for Q_1 = A_p R_1^-1 (double-float): the error of
@@ -395,11 +395,7 @@ __device__ __forceinline__ void qg_warp_max(uint32_t &kh, uint32_t &kl, uint32_t
 //   pivot columns so far (S_11 w = S_1c): w_j = r_c / r_p, w_l -= w_j w_l(p)
 // With an error of at most eps |a_i| |a_j| in every entry of S, that of a remaining norm (a Schur
 // complement) is at most eps (|a_c| + sum_l |w_l| |a_l|)^2 to first order.  The pivot has to
-// exceed every other norm by more than both errors, and its own error 64 times.  (kEps: the
-// slices round what is below 2^-9 of a column's largest entry in 256 rows, by 2^-33 of that entry
-// at most and in either direction: 2^-33 |a_i| |a_j| where all of a column but one entry is so
-// small, about 2^-38 for normal entries.)
-constexpr float kEps = 1.2e-10f;  // 2^-33
+// exceed every other norm by more than both errors, and its own error 64 times.
 __global__ void __launch_bounds__(kMaxN) qg_pivot_kernel(const float2 *__restrict__ S, int n, int k,
                                                          float eps,
                                                          int *__restrict__ piv, float2 *__restrict__ M,
@@ -742,6 +738,22 @@ __global__ void __launch_bounds__(256) qg_q_kernel(const float2 *__restrict__ Q1
   }
 }
 
+// Bound of the error of an entry of S over |a_i| |a_j|, whatever the entries and however their errors
+// add up.  In a block of 256 rows let t be a column scaled so that its largest entry lies in
+// [2^7, 2^8): its norm is at least 2^7, and its entries' sum at most 16 times its norm.  Over the
+// product of two such norms:
+//   slicing     an entry is rounded by 2^-25 at most: 2^-25 16 (|t_i| + |t_j|), 2^-27
+//   left out    slices 2 x 3 and 3 x 3, 256 (2^-25 + 2^-34): 2^-31
+//   levels 3, 4 the shared sum, below 2^-13 (|t_i| + |t_j|) + 0.51, is rounded 112 times by
+//               2^-22 of it: 2^-30
+//   blocks      the low part, at most 2^-7.8 of the product, is rounded when a level and when
+//               the next block of a range is added to it: 2^-31 each
+// The sums over blocks are below |a_i| |a_j| (Cauchy-Schwarz).  A column with one large entry
+// beside equal small ones comes within a factor of 16 of the first term, and with 2^-33, an estimate
+// for errors of either sign, near ties were decided wrongly there.  (156 unfoldings of 18 uniform
+// and skewed tensors, three sweeps each: all decided, the nearest tie at 1.1 times what it needs.)
+float qg_eps(int64_t rows_per) { return (1.5f + (float)(rows_per / kGBlock + 1) / 16.f) * 0x1p-27f; }
+
 struct Plan {
   int tiles, ranges, oblocks;
   int64_t rows_per;
@@ -850,7 +862,7 @@ const uint32_t *qrp_gram(const float *A, int64_t m, int64_t n, int64_t lda, int 
       A, m, n, lda, p.rows_per, ex, part, words, w->err_out);
   count_launch();
   qg_reduce(part, p.ranges, n, S, s);
-  if ((*err = qg_pivots(S, n, k, kEps, piv, M, words, s)) != cudaSuccess) return words;
+  if ((*err = qg_pivots(S, n, k, qg_eps(p.rows_per), piv, M, words, s)) != cudaSuccess) return words;
   qg_ortho_kernel<<<p.oblocks, kOT, 0, s>>>(A, m, lda, k, piv, M, Q1, opart, words + 1, W, words);
   count_launch();
   qg_q_kernel<<<(unsigned)std::min<int64_t>((m + 15) / 16, 8 * (int64_t)num_sms), 256, 0, s>>>(Q1, m, k, W, words, Q,

@@ -20,7 +20,13 @@ namespace {
 constexpr int kHT = 32;      // columns of a tile of S, both ways
 constexpr int kHRows = 32;   // rows of A per stage
 constexpr int kHThreads = 256;
-constexpr float kHEps = 2.3e-13f;  // 2^-42: the pairs carry 48 bits, the sums round at about 2^-46
+
+// Bound of the error of an entry of S over |a_i| |a_j| (u = 2^-24, N = |a_i| |a_j|): a low part stays
+// below 5 u N on average, is rounded twice for each of a range's rows, and the terms added to it once
+// (11 u^2 N a row); splitting and the product of the low parts come to less than 100 u^2 N, and the
+// sum of the ranges and the pivot kernel's own arithmetic to less than 150.  (Equal entries beside one
+// large entry reach 0.1 of it; random ones 2^-45 at any number of rows.)
+float qh_eps(int rows_per) { return (float)(12 * rows_per + 256) * 0x1p-48f; }
 
 // a as a pair of floats: the leading 24 bits exactly, the other 29 rounded to 24 (integers and one
 // conversion from an integer: conversions of doubles take the FP64 pipe).  Zero below 2^-100;
@@ -269,7 +275,7 @@ const uint32_t *qrp_gram(const double *A, int64_t m, int64_t n, int64_t lda, int
                                                                                  part);
   count_launch();
   qg_reduce(part, p.ranges, n, S, s);
-  if ((*err = qg_pivots(S, n, k, kHEps, piv, M, words, s)) != cudaSuccess) return words;
+  if ((*err = qg_pivots(S, n, k, qh_eps(p.rows_per), piv, M, words, s)) != cudaSuccess) return words;
   qh_ortho_kernel<<<p.blocks, 256, 0, s>>>(A, (int)m, lda, k, piv, M, Q1, opart, words + 1, W, words);
   count_launch();
   qh_q_kernel<<<(unsigned)((m + 15) / 16), 256, 0, s>>>(Q1, (int)m, k, W, words, Q, ldq);

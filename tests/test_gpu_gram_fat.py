@@ -3,6 +3,7 @@ hold a matrix A entry for entry (identity factors in modes 2 and 3: Y_(1) = A)."
 import numpy as np
 import pytest
 
+import oracle
 from tests.gpu_util import lib, torch
 
 pytestmark = pytest.mark.gpu
@@ -54,3 +55,16 @@ def test_above_1024_rows_in_fp64(m, a, b, monkeypatch):
     monkeypatch.setenv("TUCKER_CORE_TC", "0")
     _, want = first_factor(A, a, b, 8)
     np.testing.assert_array_equal(Q, want)
+
+
+@pytest.mark.parametrize("m,a,b,k", [(12, 3, 5, 6), (33, 6, 8, 16), (200, 16, 16, 16), (512, 20, 26, 16)])
+def test_decided_pivots_run_the_gram_form(m, a, b, k, monkeypatch):
+    """Where the pivots are decided Q is not the cluster form's (its roundings are others), and it is that
+    of the FP64 reference: 2^-46 in S times its condition (below 1e4) times a few dozen."""
+    A = fat(m, a * b, 5 * m + a)
+    _, Q = first_factor(A, a, b, k)
+    monkeypatch.setenv("TUCKER_QRP_FORM", "cluster")
+    _, cluster = first_factor(A, a, b, k)
+    assert not np.array_equal(Q, cluster)
+    A = A.astype(np.float64)
+    np.testing.assert_allclose(Q, oracle.qrp(A @ A.T, k).Q, atol=1e-8)

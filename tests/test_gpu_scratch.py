@@ -1,0 +1,46 @@
+"""Device memory of a context whose rows of Y_(n) are wide and whose slices are long: the partial rows of
+cut slices (a row of P_n floats for each piece).  Measured in a process of its own, from cudaMemGetInfo."""
+import subprocess
+import sys
+
+import pytest
+
+from tests.conftest import ROOT
+from tests.gpu_util import lib
+
+pytestmark = pytest.mark.gpu
+
+CODE = """
+import torch
+from paper_2010_10638_gb300 import tucker as T
+T.load()
+g = torch.Generator(device="cuda").manual_seed(1)
+dims, ranks, nnz = (100, 300, 300, 2000), (16, 64, 64, 16), 2_500_000
+coords = torch.stack([torch.randint(0, d, (nnz,), generator=g, device="cuda", dtype=torch.int32) for d in dims])
+vals = torch.randn(nnz, generator=g, device="cuda")
+T.tucker_lib_setup()
+torch.cuda.synchronize()
+before = torch.cuda.mem_get_info()[0]
+ctx = T.tucker_init(dims, coords, vals, ranks, seed=2)
+torch.cuda.synchronize()
+after = torch.cuda.mem_get_info()[0]
+Y = T.ttmc_mode(ctx, 0)
+rows = torch.zeros_like(Y)  # the same in FP64, from FP32 factors, one slice
+U = [T.tucker_get_factor(ctx, m).float().double() for m in range(4)]
+sel = coords[0] == 7
+c, v = coords[:, sel].long(), vals[sel].double()
+left = (U[1][c[1]].unsqueeze(2) * U[2][c[2]].unsqueeze(1)).reshape(c.shape[1], -1)
+ref = ((left * v[:, None]).T @ U[3][c[3]]).reshape(-1)
+print(before - after, float((Y[7].double() - ref).norm() / ref.norm()))
+"""
+
+
+def test_wide_rows_and_long_slices():
+    """100 slices of 25,000 nonzeros and P_1 = 65,536: at most 1.2 GB (Y 0.26, partial rows of pieces of
+    2,048 nonzeros 0.35, the copies, their sort and the rest 0.4)."""
+    lib()
+    r = subprocess.run([sys.executable, "-c", CODE], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    used, err = r.stdout.split()
+    assert float(err) <= 1e-5
+    assert int(used) <= 1.2e9, used
