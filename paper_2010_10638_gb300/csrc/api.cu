@@ -163,7 +163,7 @@ static tucker_status init_impl(Ctx *c, const uint32_t *coords, const float *vals
   for (int n = 0; n < N; ++n) {
     const ModeCopy &mc = c->mode[n];
     ymax = std::max(ymax, mc.I * mc.P);
-    carry_max = std::max(carry_max, std::max(mc.n_units, mc.fn_units) * mc.P);
+    carry_max = std::max(carry_max, std::max(mc.n_slots, mc.fn_slots) * mc.P);
     Imax = std::max(Imax, mc.I);
     IRmax = std::max(IRmax, c->dims[n] * c->ranks[n]);
     const int ncols = qrp_n_cols(c, n);
@@ -201,13 +201,13 @@ static tucker_status init_impl(Ctx *c, const uint32_t *coords, const float *vals
     }
     if (gp) TK_CUDA(dev_alloc(c, &c->gram_part, gp));
   }
-  {  // column sums of squares from the pipelined TTMc: one row per block, one per split slice
+  {  // column sums of squares from the pipelined TTMc (P_n <= 256): one row per block, one per split slice
     int64_t rows = 0, pmax = 1;
     for (int n = 0; n < N; ++n) {
       const ModeCopy &mc = c->mode[n];
       int64_t r = std::max(ttmc_pipe_blocks(mc.n_units) + mc.n_long, ttmc_pipe_blocks(mc.fn_units) + mc.fn_long);
       r += (r + 63) / 64;  // the reduction's chunk sums (64 rows each)
-      rows = std::max(rows, r * mc.P);
+      if (mc.P <= 256) rows = std::max(rows, r * mc.P);
       pmax = std::max(pmax, mc.P);
     }
     TK_CUDA(dev_alloc(c, &c->sq_part, (size_t)std::max<int64_t>(rows, 1)));

@@ -41,9 +41,10 @@ struct ModeCopy {
   int32_t *unit_slot = nullptr;        // [n_units] -1: whole slices -> Y; >= 0: partial row slot
   int64_t n_units = 0;
   uint32_t *long_k = nullptr;          // [n_long] slices longer than `chunk`
-  uint32_t *long_u0 = nullptr;         // [n_long] their first unit (= first partial slot)
+  uint32_t *long_s0 = nullptr;         // [n_long] the slot of their first partial row
   uint32_t *long_np = nullptr;         // [n_long] their number of units
   int64_t n_long = 0;
+  int64_t n_slots = 0;                 // partial rows of the long slices (some unused)
   uint32_t *src = nullptr;             // [nnz] index in the coalesced order of sorted position e;
                                        // nullptr for a mode 1 copy in the coalesced order itself
   // Fiber level (order 3): within a slice, runs of nonzeros with the same index of the
@@ -62,8 +63,8 @@ struct ModeCopy {
   uint32_t *funit_e0 = nullptr, *funit_k0 = nullptr;
   int32_t *funit_slot = nullptr;
   int64_t fn_units = 0;
-  uint32_t *flong_k = nullptr, *flong_u0 = nullptr, *flong_np = nullptr;
-  int64_t fn_long = 0;
+  uint32_t *flong_k = nullptr, *flong_s0 = nullptr, *flong_np = nullptr;
+  int64_t fn_long = 0, fn_slots = 0;
 };
 
 constexpr int kFiberCap = 32;  // nonzeros per fiber at most (longer runs are cut)
@@ -123,7 +124,7 @@ struct Ctx {
   bool tm16_ok[kMaxOrder] = {};
 
   float *Y = nullptr;          // TTMc output of the current mode (max I_n * P_n floats)
-  float *carry = nullptr;      // partial rows of split slices (max n_units * P_n floats)
+  float *carry = nullptr;      // partial rows of split slices (max n_slots * P_n floats)
   float *fib_T = nullptr;      // fiber form: factor sums of the fibers (max F * R_last floats)
   uint32_t *fib_iota = nullptr;  // fiber form: 0, 1, ..., F-1 (max F)
   float *fib_ones = nullptr;   // fiber form: 1.0f (max F)

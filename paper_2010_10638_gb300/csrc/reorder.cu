@@ -752,8 +752,8 @@ __global__ void __launch_bounds__(1024) unit_scan_kernel(int64_t S, const uint32
 
 __global__ void unit_write_kernel(int64_t S, const uint32_t *sptr, const uint32_t *nu,
                                   const uint32_t *uoff, const uint32_t *islong, const uint32_t *lid,
-                                  uint32_t *unit_e0, uint32_t *unit_k0, int32_t *unit_slot, uint32_t *long_k,
-                                  uint32_t *long_u0, uint32_t *long_np) {
+                                  uint32_t chunk, uint32_t *unit_e0, uint32_t *unit_k0, int32_t *unit_slot,
+                                  uint32_t *long_k, uint32_t *long_s0, uint32_t *long_np) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < S; k += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t n = nu[k];
     if (n == 0) continue;
@@ -761,7 +761,7 @@ __global__ void unit_write_kernel(int64_t S, const uint32_t *sptr, const uint32_
     if (islong[k]) {  // its pieces: unit_long_kernel
       const uint32_t l = lid[k];
       long_k[l] = (uint32_t)k;
-      long_u0[l] = u0;
+      long_s0[l] = sptr[k] / chunk + l;
       long_np[l] = n;
     } else {
       unit_e0[u0] = sptr[k];
@@ -771,16 +771,19 @@ __global__ void unit_write_kernel(int64_t S, const uint32_t *sptr, const uint32_
   }
 }
 
-// the units of the long slices, one block per slice at a time
-__global__ void unit_long_kernel(int64_t n_long, const uint32_t *long_k, const uint32_t *long_u0,
-                                 const uint32_t *long_np, const uint32_t *sptr, uint32_t chunk, uint32_t *unit_e0,
-                                 uint32_t *unit_k0, int32_t *unit_slot) {
+// The units of the long slices, one block per slice at a time.  Only these have a partial row: piece p of
+// long slice l, from position e0 on, has slot e0 / chunk + l + p.  (A slice's pieces start `chunk` apart, and
+// the next long slice has a larger l and starts no lower, so no two pieces share a slot, and all slots lie
+// below (positions - 1) / chunk + n_long; no scan of the long slices' pieces is needed.)
+__global__ void unit_long_kernel(int64_t n_long, const uint32_t *long_k, const uint32_t *long_s0,
+                                 const uint32_t *long_np, const uint32_t *uoff, const uint32_t *sptr, uint32_t chunk,
+                                 uint32_t *unit_e0, uint32_t *unit_k0, int32_t *unit_slot) {
   for (int64_t l = blockIdx.x; l < n_long; l += gridDim.x) {
-    const uint32_t k = long_k[l], u0 = long_u0[l], np = long_np[l], e0 = sptr[k];
+    const uint32_t k = long_k[l], u0 = uoff[k], s0 = long_s0[l], np = long_np[l], e0 = sptr[k];
     for (uint32_t p = threadIdx.x; p < np; p += blockDim.x) {
       unit_e0[u0 + p] = e0 + p * chunk;
       unit_k0[u0 + p] = k;
-      unit_slot[u0 + p] = (int32_t)(u0 + p);
+      unit_slot[u0 + p] = (int32_t)(s0 + p);
     }
   }
 }
@@ -797,11 +800,13 @@ __global__ void unit_long_kernel(int64_t n_long, const uint32_t *long_k, const u
 //           589,320 nonzeros in 43 to 1,678 slices, BF16, three modes 61 us, at 128 65 us), and
 //           1.5 times the mode's average slice up to 256: slices of about the same length stay
 //           whole, which saves the kernel that adds the pieces (10,000 nonzeros, slices of 100:
-//           11 us a mode, cut at 64 13 us).
+//           11 us a mode, cut at 64 13 us).  Rows of Y so wide that the pieces' partial rows would take
+//           more than 256 MB: up to 2,048 while that leaves eight units per SM (a wide row's columns are
+//           work for many blocks).
 struct UnitSize {
   int chunk, run;
 };
-static UnitSize pick_units(int64_t nnz, int64_t slices, int num_sms) {
+static UnitSize pick_units(int64_t nnz, int64_t slices, int64_t P, int num_sms) {
   const char *f = std::getenv("TUCKER_TTMC_CHUNK");
   if (f) {
     int v = std::atoi(f);
@@ -813,6 +818,8 @@ static UnitSize pick_units(int64_t nnz, int64_t slices, int num_sms) {
   u.chunk = std::max(nnz >= (int64_t)num_sms * 8 * 256 ? 256 : 128, u.run);
   const int64_t whole = (3 * nnz / (2 * std::max<int64_t>(slices, 1)) + 31) / 32 * 32;
   if (whole <= 256) u.chunk = std::max(u.chunk, (int)whole);
+  const int64_t most = std::max<int64_t>(256, std::min<int64_t>(2048, nnz / ((int64_t)num_sms * 8)));
+  for (int w = 256; w <= most && nnz / u.chunk * P > (int64_t)(64 << 20); w *= 2) u.chunk = std::max(u.chunk, w);
   return u;
 }
 
@@ -856,13 +863,13 @@ static tucker_status read_u32(Ctx *c, const uint32_t *d, uint32_t *h, cudaStream
 
 // Work units over a slice table `ptr` ([S+1] offsets into positions: nonzeros or fibers).
 struct UnitTables {
-  uint32_t **e0, **k0, **long_k, **long_u0, **long_np;
+  uint32_t **e0, **k0, **long_k, **long_s0, **long_np;
   int32_t **slot;
-  int64_t *n_units, *n_long;
+  int64_t *n_units, *n_long, *n_slots;
 };
 
-static tucker_status build_units(Ctx *c, int64_t S, const uint32_t *ptr, UnitSize size, uint32_t *nu, uint32_t *islong,
-                                 uint32_t *uoff, uint32_t *lid, uint32_t *stmp, uint32_t *d_small, UnitTables o,
+static tucker_status build_units(Ctx *c, int64_t S, int64_t positions, const uint32_t *ptr, UnitSize size, uint32_t *nu,
+                                 uint32_t *islong, uint32_t *uoff, uint32_t *lid, uint32_t *stmp, uint32_t *d_small, UnitTables o,
                                  cudaStream_t s) {
   const uint32_t chunk = (uint32_t)size.chunk, run = (uint32_t)size.run;
   uint32_t nunits = 0, nlong = 0;
@@ -884,19 +891,20 @@ static tucker_status build_units(Ctx *c, int64_t S, const uint32_t *ptr, UnitSiz
   }
   *o.n_units = nunits;
   *o.n_long = nlong;
+  *o.n_slots = nlong ? (positions - 1) / size.chunk + nlong : 0;
   TK_TRY(dev_alloc(c, o.e0, (size_t)std::max<uint32_t>(nunits, 1)));
   TK_TRY(dev_alloc(c, o.k0, (size_t)std::max<uint32_t>(nunits, 1)));
   TK_TRY(dev_alloc(c, o.slot, (size_t)std::max<uint32_t>(nunits, 1)));
   TK_TRY(dev_alloc(c, o.long_k, (size_t)std::max<uint32_t>(nlong, 1)));
-  TK_TRY(dev_alloc(c, o.long_u0, (size_t)std::max<uint32_t>(nlong, 1)));
+  TK_TRY(dev_alloc(c, o.long_s0, (size_t)std::max<uint32_t>(nlong, 1)));
   TK_TRY(dev_alloc(c, o.long_np, (size_t)std::max<uint32_t>(nlong, 1)));
   if (S > 0) {
-    unit_write_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, nu, uoff, islong, lid, *o.e0, *o.k0,
-                                                   *o.slot, *o.long_k, *o.long_u0, *o.long_np);
+    unit_write_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, nu, uoff, islong, lid, chunk, *o.e0, *o.k0,
+                                                   *o.slot, *o.long_k, *o.long_s0, *o.long_np);
     ::tk::count_launch();
     if (nlong > 0) {
       unit_long_kernel<<<(unsigned)std::min<uint32_t>(nlong, (uint32_t)c->num_sms * 4), 256, 0, s>>>(
-          nlong, *o.long_k, *o.long_u0, *o.long_np, ptr, chunk, *o.e0, *o.k0, *o.slot);
+          nlong, *o.long_k, *o.long_s0, *o.long_np, uoff, ptr, chunk, *o.e0, *o.k0, *o.slot);
       ::tk::count_launch();
     }
   }
@@ -1165,11 +1173,11 @@ tucker_status build_sorted_copies(Ctx *c, const uint32_t *coords_in, const float
     }
     // work units
     {
-      UnitTables o{&mc.unit_e0, &mc.unit_k0, &mc.long_k, &mc.long_u0, &mc.long_np, &mc.unit_slot, &mc.n_units,
-                   &mc.n_long};
-      const UnitSize size = pick_units(Z, S, c->num_sms);
+      UnitTables o{&mc.unit_e0,   &mc.unit_k0, &mc.long_k, &mc.long_s0, &mc.long_np,
+                   &mc.unit_slot, &mc.n_units, &mc.n_long, &mc.n_slots};
+      const UnitSize size = pick_units(Z, S, mc.P, c->num_sms);
       mc.chunk = size.chunk;
-      tucker_status st2 = build_units(c, S, mc.sptr, size, nu, islong, uoff, lid, stmp, d_small, o, s);
+      tucker_status st2 = build_units(c, S, Z, mc.sptr, size, nu, islong, uoff, lid, stmp, d_small, o, s);
       if (st2 != TUCKER_OK) return st2;
     }
   }
@@ -1309,9 +1317,9 @@ tucker_status build_sorted_copies(Ctx *c, const uint32_t *coords_in, const float
           if (v >= 32 && v <= (1 << 20) && (v % 32) == 0) mc.fchunk = v;
         }
       }
-      UnitTables o{&mc.funit_e0, &mc.funit_k0, &mc.flong_k, &mc.flong_u0, &mc.flong_np, &mc.funit_slot,
-                   &mc.fn_units, &mc.fn_long};
-      st2 = build_units(c, mc.S, mc.fsptr, {mc.fchunk, mc.fchunk}, nu, islong, uoff, lid, stmp, d_small, o, s);
+      UnitTables o{&mc.funit_e0,   &mc.funit_k0, &mc.flong_k, &mc.flong_s0, &mc.flong_np,
+                   &mc.funit_slot, &mc.fn_units, &mc.fn_long, &mc.fn_slots};
+      st2 = build_units(c, mc.S, F, mc.fsptr, {mc.fchunk, mc.fchunk}, nu, islong, uoff, lid, stmp, d_small, o, s);
       if (st2 != TUCKER_OK) return st2;
     } else {  // the nonzero form does not depend on the order within a slice
       mc.fmid_t = 0;

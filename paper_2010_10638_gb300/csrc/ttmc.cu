@@ -1348,17 +1348,17 @@ __global__ void __launch_bounds__(kTmaWarps * 32) ttmc_bf16_tma_kernel(const Ttm
 // reproducible, and a slice cut into thousands of pieces is summed by many blocks.  With
 // `sq` given, the exact square of each finished entry goes to sq[l * P + c] as a pair.
 constexpr int kFixWarps = 8;
-__global__ void __launch_bounds__(kFixWarps * 32) ttmc_fixup_kernel(const uint32_t *long_k, const uint32_t *long_u0,
+__global__ void __launch_bounds__(kFixWarps * 32) ttmc_fixup_kernel(const uint32_t *long_k, const uint32_t *long_s0,
                                                                      const uint32_t *long_np, const uint32_t *sid,
                                                                      const float *carry, float *Y, int64_t P,
                                                                      float2 *sq) {
   __shared__ float part[kFixWarps][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t l = blockIdx.x, c = (int64_t)blockIdx.y * 32 + lane;
-  const uint32_t row = __ldg(sid + __ldg(long_k + l)), u0 = __ldg(long_u0 + l), np = __ldg(long_np + l);
+  const uint32_t row = __ldg(sid + __ldg(long_k + l)), s0 = __ldg(long_s0 + l), np = __ldg(long_np + l);
   float s = 0.f;
   if (c < P) {
-    const float *base = carry + (size_t)u0 * P + c;
+    const float *base = carry + (size_t)s0 * P + c;
     uint32_t q = (uint32_t)warp;
     for (; q + 3u * kFixWarps < np; q += 4u * kFixWarps) {
       float v[4];
@@ -1383,11 +1383,11 @@ __global__ void __launch_bounds__(kFixWarps * 32) ttmc_fixup_kernel(const uint32
   }
 }
 
-static void launch_fixup(const uint32_t *long_k, const uint32_t *long_u0, const uint32_t *long_np, int64_t n_long,
+static void launch_fixup(const uint32_t *long_k, const uint32_t *long_s0, const uint32_t *long_np, int64_t n_long,
                          const uint32_t *sid, const float *carry, float *Y, int64_t P, cudaStream_t s,
                          float2 *sq = nullptr) {
   const dim3 grid((unsigned)n_long, (unsigned)((P + 31) / 32));
-  ttmc_fixup_kernel<<<grid, kFixWarps * 32, 0, s>>>(long_k, long_u0, long_np, sid, carry, Y, P, sq);
+  ttmc_fixup_kernel<<<grid, kFixWarps * 32, 0, s>>>(long_k, long_s0, long_np, sid, carry, Y, P, sq);
   ::tk::count_launch();
 }
 
@@ -1674,7 +1674,7 @@ bool ttmc_tiled(const Ctx *c, int mode) {
 // What the nonzero forms leave to do: rows of slices cut over several units, empty rows.
 void ttmc_finish(Ctx *c, int mode, float *Y, float2 *sq, cudaStream_t s) {
   const ModeCopy &mc = c->mode[mode];
-  if (mc.n_long > 0) launch_fixup(mc.long_k, mc.long_u0, mc.long_np, mc.n_long, mc.sid, c->carry, Y, mc.P, s, sq);
+  if (mc.n_long > 0) launch_fixup(mc.long_k, mc.long_s0, mc.long_np, mc.n_long, mc.sid, c->carry, Y, mc.P, s, sq);
   if (mc.n_empty > 0) {
     ttmc_zero_rows_kernel<<<(unsigned)std::min<int64_t>(mc.n_empty, 65535), 256, 0, s>>>(mc.empty, mc.n_empty, Y,
                                                                                         mc.P);
@@ -1781,7 +1781,7 @@ static tucker_status ttmc_impl(Ctx *c, int mode, float *Y, const float *val, con
       dispatch_pipe(r, s, &err);  // covers the shape (checked above)
       TK_CUDA(err);
       if (mc.fn_long > 0)
-        launch_fixup(mc.flong_k, mc.flong_u0, mc.flong_np, mc.fn_long, mc.sid, c->carry, Y, mc.P, s,
+        launch_fixup(mc.flong_k, mc.flong_s0, mc.flong_np, mc.fn_long, mc.sid, c->carry, Y, mc.P, s,
                      sq ? c->sq_part + nb * mc.P : nullptr);
       if (sq) {
         launch_colsq(c->sq_part, nb + mc.fn_long, mc.P, c->sq_cnt, colsq, s);
