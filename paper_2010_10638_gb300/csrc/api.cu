@@ -216,18 +216,6 @@ static tucker_status init_impl(Ctx *c, const uint32_t *coords, const float *vals
     TK_CUDA(cudaMemsetAsync(c->sq_cnt, 0, 8 * sizeof(unsigned), s));
     c->sq_elems = rows;
   }
-  for (int n = 0; n < N; ++n)
-  {
-    const int64_t I = c->mode[n].I, P = c->mode[n].P;
-    const bool fat = qrp_n_cols(c, n) == I && P > I;
-    c->qgram_bytes = std::max(c->qgram_bytes, fat ? qrp_gram_bytes64(I, I, c->ranks[n], c->num_sms)
-                                                  : qrp_gram_bytes(I, P, c->ranks[n], c->num_sms));
-  }
-  if (c->qgram_bytes && dev_alloc(c, &c->qgram, c->qgram_bytes) != cudaSuccess) {  // not needed: the cluster form
-    cudaGetLastError();
-    c->qgram = nullptr;
-    c->qgram_bytes = 0;
-  }
   TK_CUDA(dev_alloc(c, &c->G, (size_t)PR));
   TK_CUDA(dev_alloc(c, &c->core_part, core_part_elems(c->num_sms, c->mode[N - 1].P, c->ranks[N - 1])));
   TK_CUDA(dev_alloc(c, &c->core_counter, 4));
@@ -269,6 +257,19 @@ static tucker_status init_impl(Ctx *c, const uint32_t *coords, const float *vals
   }
   for (int m = 0; m < N; ++m) refresh_factor_copies(c, m, s);
   if (c->flags & TUCKER_F_BF16_FACTORS) make_factor_maps(c);
+  // the Gram forms' workspace, last: without it the cluster form runs, so it takes no memory that
+  // anything above needs
+  for (int n = 0; n < N; ++n) {
+    const int64_t I = c->mode[n].I, P = c->mode[n].P;
+    const bool fat = qrp_n_cols(c, n) == I && P > I;
+    c->qgram_bytes = std::max(c->qgram_bytes, fat ? qrp_gram_bytes64(I, I, c->ranks[n], c->num_sms)
+                                                  : qrp_gram_bytes(I, P, c->ranks[n], c->num_sms));
+  }
+  if (c->qgram_bytes && dev_alloc(c, &c->qgram, c->qgram_bytes) != cudaSuccess) {
+    cudaGetLastError();
+    c->qgram = nullptr;
+    c->qgram_bytes = 0;
+  }
   TK_CUDA(cudaGetLastError());
   TK_CUDA(cudaStreamSynchronize(s));
   c->astream = 0;  // the caller may destroy s; later allocations name their own stream

@@ -1,10 +1,12 @@
-"""Device memory of a context whose rows of Y_(n) are wide and whose slices are long: the partial rows of
-cut slices (a row of P_n floats for each piece).  Measured in a process of its own, from cudaMemGetInfo."""
+"""Device memory of a context: what it takes where rows of Y_(n) are wide and slices long (the partial rows
+of cut slices, P_n floats for each piece; measured in a process of its own, from cudaMemGetInfo), and what
+runs without the part of it that is optional."""
 import subprocess
 import sys
 
 import pytest
 
+from paper_2010_10638_gb300 import synth
 from tests.conftest import ROOT
 from tests.gpu_util import lib
 
@@ -45,3 +47,30 @@ def test_wide_rows_and_long_slices():
     used, err = r.stdout.split()
     assert float(err) <= 1e-5
     assert int(used) <= 2.34e9, used
+
+
+def test_the_optional_workspace_is_allocated_last(monkeypatch):
+    """Of the allocations of tucker_init only the last, the workspace of the QRP's Gram form, may fail
+    without the call failing: it takes no memory that another one needs.  Without it a sweep is that of
+    the cluster form, bit for bit."""
+    T = lib()
+    w = synth.make("tiny-100^3")
+    args = w.workload.dims, w.coords, w.vals, w.workload.ranks, w.U0
+    worked = []
+    for k in range(1, 200):
+        monkeypatch.setenv("TUCKER_FAIL_ALLOC_AT", str(k))
+        try:
+            ctx = T.tucker_init(*args)
+        except T.TuckerError as e:
+            assert e.name == "TUCKER_ENOMEM"
+            worked.append(False)
+        else:
+            if not any(worked):
+                fit = T.hooi_iter(ctx)
+            worked.append(True)
+            T.tucker_free(ctx)
+    first = worked.index(True)
+    assert 20 < first and all(worked[first:])
+    monkeypatch.delenv("TUCKER_FAIL_ALLOC_AT")
+    monkeypatch.setenv("TUCKER_QRP_FORM", "cluster")
+    assert T.hooi_iter(T.tucker_init(*args)) == fit
