@@ -133,9 +133,13 @@ __global__ void __launch_bounds__(kGT + 32, 1) qg_gram_kernel(const float *__res
       reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(qg_raw) + 127) & ~static_cast<uintptr_t>(127));
   // full[stage], empty[stage], levels of a block complete, levels read
   __shared__ __align__(8) unsigned long long bars[2 * kGStages + 2];
-  __shared__ uint32_t tbase;
-  if (*flag) return;  // (set by the kernel before this one; this one sets it on a timeout only)
+  __shared__ uint32_t tbase, given_up;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // (one thread reads it for all: a block that times out may set it meanwhile, and a block has to
+  // leave, or come to the allocation and the barriers below, as a whole)
+  if (tid == 0) given_up = *flag;
+  __syncthreads();
+  if (given_up) return;
   int ti = 0, tj = (int)blockIdx.x;  // tiles on and below the diagonal
   while (tj > ti) tj -= ++ti;
   const bool diag = ti == tj;

@@ -59,3 +59,14 @@ def test_separated_pivots_are_decided(m, a, b, k, monkeypatch):
     _, want = first_factor(A, a, b, k)
     assert not np.array_equal(Q, want)
     np.testing.assert_allclose(Q, want, atol=1e-5)
+
+
+def test_given_up_before_s(monkeypatch):
+    """Magnitudes outside the range: every block of S (three tiles, several ranges of rows) leaves as a whole,
+    and the cluster form runs."""
+    A = matrix(1000, 256, 2)
+    A[500, 200] *= np.float32(2.0**60)
+    _, Q = first_factor(A, 16, 16, 16)
+    monkeypatch.setenv("TUCKER_QRP_FORM", "cluster")
+    _, want = first_factor(A, 16, 16, 16)
+    np.testing.assert_array_equal(Q, want)
