@@ -44,6 +44,8 @@ struct ModeCopy {
   uint32_t *long_s0 = nullptr;         // [n_long] the slot of their first partial row
   uint32_t *long_np = nullptr;         // [n_long] their number of units
   int64_t n_long = 0;
+  uint32_t *big = nullptr;             // [n_big] those of them (0 .. n_long - 1) in more than kFixAlone pieces
+  int64_t n_big = 0;
   int64_t n_slots = 0;                 // partial rows of the long slices (some unused)
   uint32_t *src = nullptr;             // [nnz] index in the coalesced order of sorted position e;
                                        // nullptr for a mode 1 copy in the coalesced order itself
@@ -63,10 +65,11 @@ struct ModeCopy {
   uint32_t *funit_e0 = nullptr, *funit_k0 = nullptr;
   int32_t *funit_slot = nullptr;
   int64_t fn_units = 0;
-  uint32_t *flong_k = nullptr, *flong_s0 = nullptr, *flong_np = nullptr;
-  int64_t fn_long = 0, fn_slots = 0;
+  uint32_t *flong_k = nullptr, *flong_s0 = nullptr, *flong_np = nullptr, *fbig = nullptr;
+  int64_t fn_long = 0, fn_big = 0, fn_slots = 0;
 };
 
+constexpr uint32_t kFixAlone = 16;  // pieces of a cut slice that one warp adds by itself
 constexpr int kFiberCap = 32;  // nonzeros per fiber at most (longer runs are cut)
 
 // Workspace of the QR with column pivoting (one set, sized for the largest mode).

@@ -661,9 +661,10 @@ __global__ void unit_fiber_kernel(int64_t n_units, const uint32_t *unit_e0, cons
 
 // units contributed by each non-empty slice k: pieces of a long slice, or 1 for the
 // first slice of a run of short slices (a new run starts at a long slice, after a long
-// slice, and where the slice start crosses into a new multiple of `run`).
+// slice, and where the slice start crosses into a new multiple of `run`).  *nbig: += the long
+// slices of more than kFixAlone pieces.
 __global__ void unit_count_kernel(int64_t S, const uint32_t *sptr, uint32_t chunk, uint32_t run, uint32_t *nu,
-                                  uint32_t *islong) {
+                                  uint32_t *islong, uint32_t *nbig) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < S; k += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t b = sptr[k], len = sptr[k + 1] - b;
     const bool lng = len > chunk;
@@ -674,11 +675,12 @@ __global__ void unit_count_kernel(int64_t S, const uint32_t *sptr, uint32_t chun
     }
     nu[k] = lng ? (len + chunk - 1) / chunk : (head ? 1u : 0u);
     islong[k] = lng ? 1u : 0u;
+    if (nu[k] > kFixAlone) atomicAdd(nbig, 1u);
   }
 }
 
 // unit_count_kernel and the exclusive scans of both its lists in one block (total[0], total[1]:
-// their sums); up to kUnitScanMax slices, 4,096 a round (50,000 slices: 20 us as one launch,
+// their sums, total[2]: nbig, total[3]: zero); up to kUnitScanMax slices, 4,096 a round (50,000 slices: 20 us as one launch,
 // against seven launches)
 constexpr int64_t kUnitScanMax = 1 << 16;
 __global__ void __launch_bounds__(1024) unit_scan_kernel(int64_t S, const uint32_t *__restrict__ sptr, uint32_t chunk,
@@ -686,6 +688,9 @@ __global__ void __launch_bounds__(1024) unit_scan_kernel(int64_t S, const uint32
                                                          uint32_t *__restrict__ islong, uint32_t *__restrict__ uoff,
                                                          uint32_t *__restrict__ lid, uint32_t *__restrict__ total) {
   __shared__ unsigned long long wsum[32];
+  __shared__ uint32_t nbig;
+  if (threadIdx.x == 0) nbig = 0u;
+  uint32_t mine = 0u;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   unsigned long long carry = 0;  // units in the low word, long slices in the high one
   for (int64_t k0 = 0; k0 < S; k0 += 4096) {
@@ -707,6 +712,7 @@ __global__ void __launch_bounds__(1024) unit_scan_kernel(int64_t S, const uint32
         l[i] = len > chunk ? 1u : 0u;
         const bool head = k == 0 || l[i] || b - pb > chunk || b / run != pb / run;
         n[i] = l[i] ? (len + chunk - 1) / chunk : (head ? 1u : 0u);
+        mine += n[i] > kFixAlone ? 1u : 0u;
       }
       sum += n[i] + ((unsigned long long)l[i] << 32);
     }
@@ -744,16 +750,21 @@ __global__ void __launch_bounds__(1024) unit_scan_kernel(int64_t S, const uint32
     }
     __syncthreads();  // wsum is read
   }
+  if (mine) atomicAdd(&nbig, mine);
+  __syncthreads();
   if (threadIdx.x == 0) {
     total[0] = (uint32_t)carry;
     total[1] = (uint32_t)(carry >> 32);
+    total[2] = nbig;
+    total[3] = 0u;
   }
 }
 
 __global__ void unit_write_kernel(int64_t S, const uint32_t *sptr, const uint32_t *nu,
                                   const uint32_t *uoff, const uint32_t *islong, const uint32_t *lid,
                                   uint32_t chunk, uint32_t *unit_e0, uint32_t *unit_k0, int32_t *unit_slot,
-                                  uint32_t *long_k, uint32_t *long_s0, uint32_t *long_np) {
+                                  uint32_t *long_k, uint32_t *long_s0, uint32_t *long_np, uint32_t *big,
+                                  uint32_t *nbig) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < S; k += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t n = nu[k];
     if (n == 0) continue;
@@ -763,6 +774,7 @@ __global__ void unit_write_kernel(int64_t S, const uint32_t *sptr, const uint32_
       long_k[l] = (uint32_t)k;
       long_s0[l] = sptr[k] / chunk + l;
       long_np[l] = n;
+      if (n > kFixAlone) big[atomicAdd(nbig, 1u)] = l;  // (in any order: it tells which block adds a slice up)
     } else {
       unit_e0[u0] = sptr[k];
       unit_k0[u0] = (uint32_t)k;
@@ -863,34 +875,38 @@ static tucker_status read_u32(Ctx *c, const uint32_t *d, uint32_t *h, cudaStream
 
 // Work units over a slice table `ptr` ([S+1] offsets into positions: nonzeros or fibers).
 struct UnitTables {
-  uint32_t **e0, **k0, **long_k, **long_s0, **long_np;
+  uint32_t **e0, **k0, **long_k, **long_s0, **long_np, **big;
   int32_t **slot;
-  int64_t *n_units, *n_long, *n_slots;
+  int64_t *n_units, *n_long, *n_big, *n_slots;
 };
 
 static tucker_status build_units(Ctx *c, int64_t S, int64_t positions, const uint32_t *ptr, UnitSize size, uint32_t *nu,
                                  uint32_t *islong, uint32_t *uoff, uint32_t *lid, uint32_t *stmp, uint32_t *d_small, UnitTables o,
                                  cudaStream_t s) {
   const uint32_t chunk = (uint32_t)size.chunk, run = (uint32_t)size.run;
-  uint32_t nunits = 0, nlong = 0;
+  uint32_t nunits = 0, nlong = 0, nbig = 0;
+  uint32_t *total = d_small + 2;  // units, long slices, those in many pieces, a counter for their list
   if (S > 0) {
     if (S <= kUnitScanMax) {
-      unit_scan_kernel<<<1, 1024, 0, s>>>(S, ptr, chunk, run, nu, islong, uoff, lid, d_small + 2);
+      unit_scan_kernel<<<1, 1024, 0, s>>>(S, ptr, chunk, run, nu, islong, uoff, lid, total);
       ::tk::count_launch();
     } else {
-      unit_count_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, chunk, run, nu, islong);
+      TK_TRY(cudaMemsetAsync(total, 0, 4 * sizeof(uint32_t), s));
+      unit_count_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, chunk, run, nu, islong, total + 2);
       ::tk::count_launch();
-      exclusive_scan_total(nu, uoff, S, stmp, d_small + 2, s);
-      exclusive_scan_total(islong, lid, S, stmp, d_small + 3, s);
+      exclusive_scan_total(nu, uoff, S, stmp, total, s);
+      exclusive_scan_total(islong, lid, S, stmp, total + 1, s);
     }
-    uint32_t h2[2];
-    TK_TRY(cudaMemcpyAsync(h2, d_small + 2, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    uint32_t h[3];
+    TK_TRY(cudaMemcpyAsync(h, total, 3 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     TK_TRY(cudaStreamSynchronize(s));
-    nunits = h2[0];
-    nlong = h2[1];
+    nunits = h[0];
+    nlong = h[1];
+    nbig = h[2];
   }
   *o.n_units = nunits;
   *o.n_long = nlong;
+  *o.n_big = nbig;
   *o.n_slots = nlong ? (positions - 1) / size.chunk + nlong : 0;
   TK_TRY(dev_alloc(c, o.e0, (size_t)std::max<uint32_t>(nunits, 1)));
   TK_TRY(dev_alloc(c, o.k0, (size_t)std::max<uint32_t>(nunits, 1)));
@@ -898,9 +914,10 @@ static tucker_status build_units(Ctx *c, int64_t S, int64_t positions, const uin
   TK_TRY(dev_alloc(c, o.long_k, (size_t)std::max<uint32_t>(nlong, 1)));
   TK_TRY(dev_alloc(c, o.long_s0, (size_t)std::max<uint32_t>(nlong, 1)));
   TK_TRY(dev_alloc(c, o.long_np, (size_t)std::max<uint32_t>(nlong, 1)));
+  if (nbig) TK_TRY(dev_alloc(c, o.big, (size_t)nbig));
   if (S > 0) {
     unit_write_kernel<<<grid_for(S), 256, 0, s>>>(S, ptr, nu, uoff, islong, lid, chunk, *o.e0, *o.k0,
-                                                   *o.slot, *o.long_k, *o.long_s0, *o.long_np);
+                                                   *o.slot, *o.long_k, *o.long_s0, *o.long_np, *o.big, total + 3);
     ::tk::count_launch();
     if (nlong > 0) {
       unit_long_kernel<<<(unsigned)std::min<uint32_t>(nlong, (uint32_t)c->num_sms * 4), 256, 0, s>>>(
@@ -1173,8 +1190,8 @@ tucker_status build_sorted_copies(Ctx *c, const uint32_t *coords_in, const float
     }
     // work units
     {
-      UnitTables o{&mc.unit_e0,   &mc.unit_k0, &mc.long_k, &mc.long_s0, &mc.long_np,
-                   &mc.unit_slot, &mc.n_units, &mc.n_long, &mc.n_slots};
+      UnitTables o{&mc.unit_e0,   &mc.unit_k0, &mc.long_k, &mc.long_s0, &mc.long_np, &mc.big,
+                   &mc.unit_slot, &mc.n_units, &mc.n_long, &mc.n_big,   &mc.n_slots};
       const UnitSize size = pick_units(Z, S, mc.P, c->num_sms);
       mc.chunk = size.chunk;
       tucker_status st2 = build_units(c, S, Z, mc.sptr, size, nu, islong, uoff, lid, stmp, d_small, o, s);
@@ -1317,8 +1334,8 @@ tucker_status build_sorted_copies(Ctx *c, const uint32_t *coords_in, const float
           if (v >= 32 && v <= (1 << 20) && (v % 32) == 0) mc.fchunk = v;
         }
       }
-      UnitTables o{&mc.funit_e0,   &mc.funit_k0, &mc.flong_k, &mc.flong_s0, &mc.flong_np,
-                   &mc.funit_slot, &mc.fn_units, &mc.fn_long, &mc.fn_slots};
+      UnitTables o{&mc.funit_e0,   &mc.funit_k0, &mc.flong_k, &mc.flong_s0, &mc.flong_np, &mc.fbig,
+                   &mc.funit_slot, &mc.fn_units, &mc.fn_long, &mc.fn_big,   &mc.fn_slots};
       st2 = build_units(c, mc.S, F, mc.fsptr, {mc.fchunk, mc.fchunk}, nu, islong, uoff, lid, stmp, d_small, o, s);
       if (st2 != TUCKER_OK) return st2;
     } else {  // the nonzero form does not depend on the order within a slice

@@ -1342,52 +1342,117 @@ __global__ void __launch_bounds__(kTmaWarps * 32) ttmc_bf16_tma_kernel(const Ttm
   }
 }
 
-// Rows of slices split over several units: block (l, c) sums the partial rows of long
-// slice l for columns [32c, 32c + 32).  Warp w adds the pieces w, w + 8, ... (four loads in
-// flight), then the eight warp sums are added in warp order: a fixed order, so Y is
-// reproducible, and a slice cut into thousands of pieces is summed by many blocks.  With
-// `sq` given, the exact square of each finished entry goes to sq[l * P + c] as a pair.
+// Rows of slices split over several units; all sums in a fixed order, so Y is reproducible: the pieces
+// w, w + 8, ... give sum w, and the eight sums are added in order.  Up to kFixAlone pieces: one warp for
+// 128 columns of a slice (32 where P is not a multiple of 4).  More: a block for 32 columns (the first blocks
+// of the grid, by the list of these slices), warp w forming sum w.  With `sq` given, the exact square of each
+// finished entry goes to sq[l * P + c] as a pair.
+// Most slices that are cut are a little longer than a unit: as blocks for 32 columns, most of the warps
+// without a piece, 3,000 slices of two pieces of 1,024 columns took 93 us, twice the TTMc itself, and with
+// it more than in coarser units (1M nonzeros, ranks 32^3, BF16, three modes 172 -> 270 us); now 135 us.
+// Slices of many pieces need the blocks: by warps, 200 slices of 100 pieces on average, of 64 columns,
+// took 20 us instead of 6.  32 registers a thread: latency bounds both, so an SM has to hold its 64 warps
+// (200 slices of 20 pieces, 512 columns: 11 us, with 48 registers 14).
 constexpr int kFixWarps = 8;
-__global__ void __launch_bounds__(kFixWarps * 32) ttmc_fixup_kernel(const uint32_t *long_k, const uint32_t *long_s0,
-                                                                     const uint32_t *long_np, const uint32_t *sid,
-                                                                     const float *carry, float *Y, int64_t P,
-                                                                     float2 *sq) {
-  __shared__ float part[kFixWarps][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t l = blockIdx.x, c = (int64_t)blockIdx.y * 32 + lane;
-  const uint32_t row = __ldg(sid + __ldg(long_k + l)), s0 = __ldg(long_s0 + l), np = __ldg(long_np + l);
-  float s = 0.f;
-  if (c < P) {
-    const float *base = carry + (size_t)s0 * P + c;
-    uint32_t q = (uint32_t)warp;
-    for (; q + 3u * kFixWarps < np; q += 4u * kFixWarps) {
-      float v[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = __ldcg(base + (size_t)(q + k * kFixWarps) * P);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) s += v[k];
-    }
-    for (; q < np; q += kFixWarps) s += __ldcg(base + (size_t)q * P);
+template <int V>
+__device__ __forceinline__ void fix_load(const float *p, float (&v)[V]) {
+  if constexpr (V == 4) {
+    const float4 q = __ldcg(reinterpret_cast<const float4 *>(p));
+    v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+  } else {
+    v[0] = __ldcg(p);
   }
-  part[warp][lane] = s;
-  __syncthreads();
-  if (warp == 0 && c < P) {
-    float t = part[0][lane];
+}
+template <int V>
+__device__ __forceinline__ void fix_store(const float (&t)[V], float *y, float2 *sq) {
+  if constexpr (V == 4) {
+    *reinterpret_cast<float4 *>(y) = make_float4(t[0], t[1], t[2], t[3]);
+  } else {
+    *y = t[0];
+  }
+  if (sq) {
 #pragma unroll
-    for (int k = 1; k < kFixWarps; ++k) t += part[k][lane];
-    Y[(size_t)row * P + c] = t;
-    if (sq) {
-      const float t2 = t * t;
-      sq[(size_t)l * P + c] = make_float2(t2, fmaf(t, t, -t2));
+    for (int i = 0; i < V; ++i) {
+      const float t2 = t[i] * t[i];
+      sq[i] = make_float2(t2, fmaf(t[i], t[i], -t2));
     }
   }
 }
+struct FixParams {
+  const uint32_t *long_k, *long_s0, *long_np, *big, *sid;
+  const float *carry;
+  float *Y;
+  int64_t P;
+  uint32_t n_long, n_big;            // (neighbouring blocks and warps: the same columns of other slices)
+  uint32_t big_blocks, items;        // blocks for the slices of the list; items of single warps
+  float2 *sq;
+};
+template <int V>
+__global__ void __launch_bounds__(kFixWarps * 32, 8) ttmc_fixup_kernel(const FixParams p) {
+  __shared__ float part[kFixWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t P = p.P;
+  if (blockIdx.x < p.big_blocks) {
+    const uint32_t l = __ldg(p.big + blockIdx.x % p.n_big);
+    const int64_t c = (int64_t)(blockIdx.x / p.n_big) * 32 + lane;
+    const uint32_t np = __ldg(p.long_np + l);
+    float s = 0.f;
+    if (c < P) {
+      const float *base = p.carry + (size_t)__ldg(p.long_s0 + l) * P + c;
+      uint32_t q = (uint32_t)warp;
+      for (; q + 3u * kFixWarps < np; q += 4u * kFixWarps) {
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = __ldcg(base + (size_t)(q + k * kFixWarps) * P);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s += v[k];
+      }
+      for (; q < np; q += kFixWarps) s += __ldcg(base + (size_t)q * P);
+    }
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && c < P) {
+      float t[1] = {part[0][lane]};
+#pragma unroll
+      for (int k = 1; k < kFixWarps; ++k) t[0] += part[k][lane];
+      fix_store<1>(t, p.Y + (size_t)__ldg(p.sid + __ldg(p.long_k + l)) * P + c, p.sq ? p.sq + (size_t)l * P + c : nullptr);
+    }
+    return;
+  }
+  const uint32_t it = (blockIdx.x - p.big_blocks) * kFixWarps + warp;
+  if (it >= p.items) return;
+  const uint32_t l = it % p.n_long, np = __ldg(p.long_np + l);
+  const int64_t c = ((int64_t)(it / p.n_long) * 32 + lane) * V;
+  if (np > kFixAlone || c >= P) return;
+  static_assert(kFixAlone == 2 * kFixWarps, "sums of at most two pieces");
+  const float *base = p.carry + (size_t)__ldg(p.long_s0 + l) * P + c;
+  float t[V] = {};
+#pragma unroll
+  for (int w0 = 0; w0 < kFixWarps; w0 += 2) {
+    if ((uint32_t)w0 >= np) break;
+    float v[4][V] = {};  // sums w0 and w0 + 1
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t q = (uint32_t)(w0 + u % 2 + u / 2 * kFixWarps);
+      if (q < np) fix_load<V>(base + (size_t)q * P, v[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+#pragma unroll
+      for (int i = 0; i < V; ++i) t[i] += v[u][i] + v[u + 2][i];
+    }
+  }
+  fix_store<V>(t, p.Y + (size_t)__ldg(p.sid + __ldg(p.long_k + l)) * P + c, p.sq ? p.sq + (size_t)l * P + c : nullptr);
+}
 
-static void launch_fixup(const uint32_t *long_k, const uint32_t *long_s0, const uint32_t *long_np, int64_t n_long,
-                         const uint32_t *sid, const float *carry, float *Y, int64_t P, cudaStream_t s,
-                         float2 *sq = nullptr) {
-  const dim3 grid((unsigned)n_long, (unsigned)((P + 31) / 32));
-  ttmc_fixup_kernel<<<grid, kFixWarps * 32, 0, s>>>(long_k, long_s0, long_np, sid, carry, Y, P, sq);
+static void launch_fixup(FixParams p, cudaStream_t s) {
+  const bool wide = p.P % 4 == 0;  // (Y and the partial rows start on 16 bytes)
+  const int64_t cols = wide ? 128 : 32;
+  // (far below 2^31: a slice in the list has more than 16 partial rows, any other two and more)
+  p.big_blocks = (uint32_t)(p.n_big * ((p.P + 31) / 32));
+  p.items = p.n_big < p.n_long ? (uint32_t)(p.n_long * ((p.P + cols - 1) / cols)) : 0u;
+  const auto kern = wide ? ttmc_fixup_kernel<4> : ttmc_fixup_kernel<1>;
+  kern<<<p.big_blocks + (p.items + kFixWarps - 1) / kFixWarps, kFixWarps * 32, 0, s>>>(p);
   ::tk::count_launch();
 }
 
@@ -1674,7 +1739,9 @@ bool ttmc_tiled(const Ctx *c, int mode) {
 // What the nonzero forms leave to do: rows of slices cut over several units, empty rows.
 void ttmc_finish(Ctx *c, int mode, float *Y, float2 *sq, cudaStream_t s) {
   const ModeCopy &mc = c->mode[mode];
-  if (mc.n_long > 0) launch_fixup(mc.long_k, mc.long_s0, mc.long_np, mc.n_long, mc.sid, c->carry, Y, mc.P, s, sq);
+  if (mc.n_long > 0)
+    launch_fixup({mc.long_k, mc.long_s0, mc.long_np, mc.big, mc.sid, c->carry, Y, mc.P, (uint32_t)mc.n_long,
+                  (uint32_t)mc.n_big, 0, 0, sq}, s);
   if (mc.n_empty > 0) {
     ttmc_zero_rows_kernel<<<(unsigned)std::min<int64_t>(mc.n_empty, 65535), 256, 0, s>>>(mc.empty, mc.n_empty, Y,
                                                                                         mc.P);
@@ -1781,8 +1848,8 @@ static tucker_status ttmc_impl(Ctx *c, int mode, float *Y, const float *val, con
       dispatch_pipe(r, s, &err);  // covers the shape (checked above)
       TK_CUDA(err);
       if (mc.fn_long > 0)
-        launch_fixup(mc.flong_k, mc.flong_s0, mc.flong_np, mc.fn_long, mc.sid, c->carry, Y, mc.P, s,
-                     sq ? c->sq_part + nb * mc.P : nullptr);
+        launch_fixup({mc.flong_k, mc.flong_s0, mc.flong_np, mc.fbig, mc.sid, c->carry, Y, mc.P, (uint32_t)mc.fn_long,
+                      (uint32_t)mc.fn_big, 0, 0, sq ? c->sq_part + nb * mc.P : nullptr}, s);
       if (sq) {
         launch_colsq(c->sq_part, nb + mc.fn_long, mc.P, c->sq_cnt, colsq, s);
         *norms = true;
