@@ -1876,6 +1876,14 @@ static tucker_status ttmc_impl(Ctx *c, int mode, float *Y, const float *val, con
       } else {
         done = dispatch_bf16(p, s, &err);
       }
+      // ranks it does not cover but the FP32 pipeline does: on the FP32 copies of the BF16 factors (plain
+      // matrices at these ranks).  1M nonzeros, ranks 8^3, three modes: 63 us; the tiled form 98, the
+      // kernel without the pipeline on BF16 rows 84
+      if (!done && p.nother == 2 && pipe_shape(p.R[0], p.R[1]) && !(c->flags & TUCKER_F_UNPIPELINED)) {
+        TtmcParams q = p;
+        for (int t = 0; t < 2; ++t) q.U[t] = c->U32[mc.other[t]];
+        done = dispatch_pipe(q, s, &err);
+      }
     } else if (!(c->flags & TUCKER_F_UNPIPELINED)) {
       const int64_t nb = ttmc_pipe_blocks(p.n_units);
       const bool sq = want_sq && pipe_shape(p.R[0], p.R[1]) && p.nother == 2 &&
