@@ -229,6 +229,7 @@ tucker_status launch_ttmc(Ctx *c, int mode, float *Y, cudaStream_t s);
 // launch_ttmc that also writes the column sums of squares of Y_(n) to colsq [P_n] where its
 // pipelined FP32 form runs (*formed true), at no extra pass over Y; *formed false otherwise.
 tucker_status launch_ttmc_norms(Ctx *c, int mode, float *Y, double *colsq, bool *formed, cudaStream_t s);
+int ttmc_units_per_sm(const Ctx *c, int mode);  // work units an SM holds, where that is what limits the TTMc; or 0
 int64_t ttmc_pipe_blocks(int64_t units);  // blocks of a pipelined TTMc launch over `units` units
 int32_t qrp_check_site();                 // checked build: first index check that failed (0: none); -1 otherwise
 // TMA descriptors of the BF16 factor copies (host only; no device work)

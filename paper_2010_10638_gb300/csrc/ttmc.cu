@@ -1581,6 +1581,16 @@ static bool tma_rows() {
   return e && e[0] == '1';
 }
 
+// The BF16 form of order 4: three blocks per SM by registers, fewer by shared memory.
+int ttmc_units_per_sm(const Ctx *c, int mode) {
+  if (!(c->flags & TUCKER_F_BF16_FACTORS) || c->N != 4) return 0;
+  const ModeCopy &mc = c->mode[mode];
+  const int R0 = c->ranks[mc.other[0]], R1 = c->ranks[mc.other[1]], RB = c->ranks[mc.other[2]];
+  if (R1 % 4 != 0 || R0 * R1 != 64 || (RB != 8 && RB != 16)) return 0;
+  const size_t smem = (size_t)kTtmcWarps * 48 * (bf16_stride(64) + bf16_stride(RB)) * sizeof(__nv_bfloat16);
+  return std::min(3, (int)(228 * 1024 / (smem + 1024))) * kTtmcWarps;
+}
+
 // BF16-factor dispatch (shapes with PL % 16 == 0 and RB % 8 == 0).
 static bool dispatch_bf16(const TtmcParams &p, cudaStream_t s, cudaError_t *err) {
   const int no = p.nother;
