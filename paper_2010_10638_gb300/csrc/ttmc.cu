@@ -1427,19 +1427,34 @@ __global__ void __launch_bounds__(kFixWarps * 32, 8) ttmc_fixup_kernel(const Fix
   static_assert(kFixAlone == 2 * kFixWarps, "sums of at most two pieces");
   const float *base = p.carry + (size_t)__ldg(p.long_s0 + l) * P + c;
   float t[V] = {};
+  if (np <= (uint32_t)kFixWarps) {  // sums of one piece
 #pragma unroll
-  for (int w0 = 0; w0 < kFixWarps; w0 += 2) {
-    if ((uint32_t)w0 >= np) break;
-    float v[4][V] = {};  // sums w0 and w0 + 1
+    for (int w0 = 0; w0 < kFixWarps; w0 += 4) {
+      if ((uint32_t)w0 >= np) break;
+      float v[4][V] = {};
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint32_t q = (uint32_t)(w0 + u % 2 + u / 2 * kFixWarps);
-      if (q < np) fix_load<V>(base + (size_t)q * P, v[u]);
+      for (int u = 0; u < 4; ++u)
+        if ((uint32_t)(w0 + u) < np) fix_load<V>(base + (size_t)(w0 + u) * P, v[u]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+#pragma unroll
+        for (int i = 0; i < V; ++i) t[i] += v[u][i];
+      }
     }
+  } else {
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
+    for (int w0 = 0; w0 < kFixWarps; w0 += 2) {  // sums w0 and w0 + 1
+      float v[4][V] = {};
 #pragma unroll
-      for (int i = 0; i < V; ++i) t[i] += v[u][i] + v[u + 2][i];
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t q = (uint32_t)(w0 + u % 2 + u / 2 * kFixWarps);
+        if (q < np) fix_load<V>(base + (size_t)q * P, v[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+#pragma unroll
+        for (int i = 0; i < V; ++i) t[i] += v[u][i] + v[u + 2][i];
+      }
     }
   }
   fix_store<V>(t, p.Y + (size_t)__ldg(p.sid + __ldg(p.long_k + l)) * P + c, p.sq ? p.sq + (size_t)l * P + c : nullptr);
