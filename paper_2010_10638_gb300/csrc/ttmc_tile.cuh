@@ -149,7 +149,6 @@ struct TileAcc {
 #pragma unroll
     for (int i = 0; i < TA; ++i) {
       const float x0 = __fmul_rn(s, a[i]);
-      
       float x1;  // (volatile: a second product, not a copy of the first)
       asm volatile("mul.rn.f32 %0, %1, %2;" : "=f"(x1) : "f"(s), "f"(a[i]));
       const TileF2 sa = tile_pack(x0, x1);

@@ -19,7 +19,7 @@ cudaError_t tile_dispatch_adj(int TA, int TB, TileParams &p, int num_sms, cudaSt
     case 2:
       TK_ADJ(2, 4, 4) TK_ADJ(2, 4, 5) TK_ADJ(2, 4, 6) TK_ADJ(2, 4, 7) TK_ADJ(2, 4, 8)
       TK_ADJ(2, 5, 4) TK_ADJ(2, 5, 5) TK_ADJ(2, 5, 6) TK_ADJ(2, 5, 7) TK_ADJ(2, 5, 8)
-      TK_ADJ(2, 6, 4) TK_ADJ(2, 6, 5) TK_ADJ(2, 6, 6) TK_ADJ(2, 6, 7) TK_ADJ(2, 6, 8) TK_ADJ(2, 6, 8)
+      TK_ADJ(2, 6, 4) TK_ADJ(2, 6, 5) TK_ADJ(2, 6, 6) TK_ADJ(2, 6, 7) TK_ADJ(2, 6, 8)
       TK_ADJ(2, 7, 4) TK_ADJ(2, 7, 5) TK_ADJ(2, 7, 6) TK_ADJ(2, 7, 7)
       TK_ADJ(2, 8, 4) TK_ADJ(2, 8, 5) TK_ADJ(2, 8, 6)
       break;
