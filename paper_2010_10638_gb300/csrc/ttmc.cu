@@ -1344,7 +1344,7 @@ __global__ void __launch_bounds__(kTmaWarps * 32) ttmc_bf16_tma_kernel(const Ttm
 
 // Rows of slices split over several units; all sums in a fixed order, so Y is reproducible: the pieces
 // w, w + 8, ... give sum w, and the eight sums are added in order.  Up to kFixAlone pieces: one warp for
-// 128 columns of a slice (32 where P is not a multiple of 4).  More: a block for 32 columns (the first blocks
+// 32 V columns of a slice.  More: a block for 32 columns (the first blocks
 // of the grid, by the list of these slices), warp w forming sum w.  With `sq` given, the exact square of each
 // finished entry goes to sq[l * P + c] as a pair.
 // Most slices that are cut are a little longer than a unit: as blocks for 32 columns, most of the warps
@@ -1359,6 +1359,9 @@ __device__ __forceinline__ void fix_load(const float *p, float (&v)[V]) {
   if constexpr (V == 4) {
     const float4 q = __ldcg(reinterpret_cast<const float4 *>(p));
     v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+  } else if constexpr (V == 2) {
+    const float2 q = __ldcg(reinterpret_cast<const float2 *>(p));
+    v[0] = q.x, v[1] = q.y;
   } else {
     v[0] = __ldcg(p);
   }
@@ -1367,6 +1370,8 @@ template <int V>
 __device__ __forceinline__ void fix_store(const float (&t)[V], float *y, float2 *sq) {
   if constexpr (V == 4) {
     *reinterpret_cast<float4 *>(y) = make_float4(t[0], t[1], t[2], t[3]);
+  } else if constexpr (V == 2) {
+    *reinterpret_cast<float2 *>(y) = make_float2(t[0], t[1]);
   } else {
     *y = t[0];
   }
@@ -1393,12 +1398,12 @@ __global__ void __launch_bounds__(kFixWarps * 32, 8) ttmc_fixup_kernel(const Fix
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t P = p.P;
   if (blockIdx.x < p.big_blocks) {
-    const uint32_t l = __ldg(p.big + blockIdx.x % p.n_big);
+    const uint32_t i = blockIdx.x % p.n_big, l = p.big ? __ldg(p.big + i) : i;
     const int64_t c = (int64_t)(blockIdx.x / p.n_big) * 32 + lane;
-    const uint32_t np = __ldg(p.long_np + l);
+    const uint32_t np = __ldg(p.long_np + l), s0 = __ldg(p.long_s0 + l), row = __ldg(p.sid + __ldg(p.long_k + l));
     float s = 0.f;
     if (c < P) {
-      const float *base = p.carry + (size_t)__ldg(p.long_s0 + l) * P + c;
+      const float *base = p.carry + (size_t)s0 * P + c;
       uint32_t q = (uint32_t)warp;
       for (; q + 3u * kFixWarps < np; q += 4u * kFixWarps) {
         float v[4];
@@ -1415,17 +1420,18 @@ __global__ void __launch_bounds__(kFixWarps * 32, 8) ttmc_fixup_kernel(const Fix
       float t[1] = {part[0][lane]};
 #pragma unroll
       for (int k = 1; k < kFixWarps; ++k) t[0] += part[k][lane];
-      fix_store<1>(t, p.Y + (size_t)__ldg(p.sid + __ldg(p.long_k + l)) * P + c, p.sq ? p.sq + (size_t)l * P + c : nullptr);
+      fix_store<1>(t, p.Y + (size_t)row * P + c, p.sq ? p.sq + (size_t)l * P + c : nullptr);
     }
     return;
   }
   const uint32_t it = (blockIdx.x - p.big_blocks) * kFixWarps + warp;
   if (it >= p.items) return;
-  const uint32_t l = it % p.n_long, np = __ldg(p.long_np + l);
+  const uint32_t l = it % p.n_long;  // (the slice's numbers are read together: a chain of reads is the time here)
+  const uint32_t np = __ldg(p.long_np + l), s0 = __ldg(p.long_s0 + l), row = __ldg(p.sid + __ldg(p.long_k + l));
   const int64_t c = ((int64_t)(it / p.n_long) * 32 + lane) * V;
   if (np > kFixAlone || c >= P) return;
   static_assert(kFixAlone == 2 * kFixWarps, "sums of at most two pieces");
-  const float *base = p.carry + (size_t)__ldg(p.long_s0 + l) * P + c;
+  const float *base = p.carry + (size_t)s0 * P + c;
   float t[V] = {};
   if (np <= (uint32_t)kFixWarps) {  // sums of one piece
 #pragma unroll
@@ -1457,16 +1463,20 @@ __global__ void __launch_bounds__(kFixWarps * 32, 8) ttmc_fixup_kernel(const Fix
       }
     }
   }
-  fix_store<V>(t, p.Y + (size_t)__ldg(p.sid + __ldg(p.long_k + l)) * P + c, p.sq ? p.sq + (size_t)l * P + c : nullptr);
+  fix_store<V>(t, p.Y + (size_t)row * P + c, p.sq ? p.sq + (size_t)l * P + c : nullptr);
 }
 
-static void launch_fixup(FixParams p, cudaStream_t s) {
-  const bool wide = p.P % 4 == 0;  // (Y and the partial rows start on 16 bytes)
-  const int64_t cols = wide ? 128 : 32;
+// V = 4 where that makes 16 warps for each SM and more (1M nonzeros, ranks 32^3, BF16: 128 us for three modes,
+// V = 2 133), else 2 (50,000 nonzeros in slices of 250 to 500, ranks 8^3: 19.9 and 21.0: V = 4 spills two
+// registers); 1 where P is odd.
+static void launch_fixup(FixParams p, int num_sms, cudaStream_t s) {
+  auto items = [&](int64_t cols) { return (uint32_t)(p.n_long * ((p.P + cols - 1) / cols)); };
+  const int V = p.P % 4 == 0 && items(128) >= 16u * (uint32_t)num_sms ? 4 : p.P % 2 == 0 ? 2 : 1;
   // (far below 2^31: a slice in the list has more than 16 partial rows, any other two and more)
   p.big_blocks = (uint32_t)(p.n_big * ((p.P + 31) / 32));
-  p.items = p.n_big < p.n_long ? (uint32_t)(p.n_long * ((p.P + cols - 1) / cols)) : 0u;
-  const auto kern = wide ? ttmc_fixup_kernel<4> : ttmc_fixup_kernel<1>;
+  p.items = p.n_big < p.n_long ? items(32 * V) : 0u;
+  if (p.n_big == p.n_long) p.big = nullptr;  // all of them: one read less in a chain of three
+  const auto kern = V == 4 ? ttmc_fixup_kernel<4> : V == 2 ? ttmc_fixup_kernel<2> : ttmc_fixup_kernel<1>;
   kern<<<p.big_blocks + (p.items + kFixWarps - 1) / kFixWarps, kFixWarps * 32, 0, s>>>(p);
   ::tk::count_launch();
 }
@@ -1766,7 +1776,7 @@ void ttmc_finish(Ctx *c, int mode, float *Y, float2 *sq, cudaStream_t s) {
   const ModeCopy &mc = c->mode[mode];
   if (mc.n_long > 0)
     launch_fixup({mc.long_k, mc.long_s0, mc.long_np, mc.big, mc.sid, c->carry, Y, mc.P, (uint32_t)mc.n_long,
-                  (uint32_t)mc.n_big, 0, 0, sq}, s);
+                  (uint32_t)mc.n_big, 0, 0, sq}, c->num_sms, s);
   if (mc.n_empty > 0) {
     ttmc_zero_rows_kernel<<<(unsigned)std::min<int64_t>(mc.n_empty, 65535), 256, 0, s>>>(mc.empty, mc.n_empty, Y,
                                                                                         mc.P);
@@ -1874,7 +1884,7 @@ static tucker_status ttmc_impl(Ctx *c, int mode, float *Y, const float *val, con
       TK_CUDA(err);
       if (mc.fn_long > 0)
         launch_fixup({mc.flong_k, mc.flong_s0, mc.flong_np, mc.fbig, mc.sid, c->carry, Y, mc.P, (uint32_t)mc.fn_long,
-                      (uint32_t)mc.fn_big, 0, 0, sq ? c->sq_part + nb * mc.P : nullptr}, s);
+                      (uint32_t)mc.fn_big, 0, 0, sq ? c->sq_part + nb * mc.P : nullptr}, c->num_sms, s);
       if (sq) {
         launch_colsq(c->sq_part, nb + mc.fn_long, mc.P, c->sq_cnt, colsq, s);
         *norms = true;

@@ -1,6 +1,7 @@
 """Rows of slices that are cut over several work units: the pieces' partial rows are added by one warp for
-each 128 or 32 columns of a row up to 16 pieces, and by a block for 32 columns for more.  Numbers of pieces
-on both sides of 8 (one round of loads) and 16, widths that are and are not multiples of 4, 32 and 128.
+each 128, 64 or 32 columns of a row up to 16 pieces, and by a block for 32 columns for more.  Numbers of pieces
+on both sides of 8 (one round of loads) and 16, widths that are and are not multiples of 2, 32 and 64; and enough
+slices for 128 columns a warp.
 
 Bar: the componentwise bound of test_gpu_ttmc_tile.py, (depth + order) 2^-24 of sum |x| prod |u|; a row of L
 nonzeros in pieces of 32 is a sum of at most 32 + L / 32 + 8 terms deep."""
@@ -43,6 +44,29 @@ def test_pieces(ranks, monkeypatch):
         assert (np.abs(Y[i + 1] - k.sum(0)) <= bound).all(), n
     assert not Y[0].any() and not Y[-1].any()
     T.tucker_free(ctx)
+
+
+@pytest.mark.parametrize("ranks", [(2, 16, 16), (2, 12, 11)], ids=lambda r: "x".join(map(str, r)))
+def test_many_slices(ranks, monkeypatch):
+    """3,000 slices of 33 to 600 nonzeros, by 128 columns a warp, against the same slices in pieces of 1,024
+    (none cut): sums of at most 600 products in other orders, each within 600 2^-24 of sum |x| prod |u|."""
+    T = lib()
+    rng = np.random.default_rng(7)
+    dims, lengths = (3000, 90, 80), rng.integers(33, 600, 3000)
+    rows = np.repeat(np.arange(3000), lengths)
+    cells = np.concatenate([rng.choice(90 * 80, n, replace=False) for n in lengths])
+    coords = torch.as_tensor(np.stack([rows, cells // 80, cells % 80]).astype(np.int32)).cuda()
+    vals = torch.as_tensor(rng.standard_normal(len(rows)).astype(np.float32)).cuda()
+    U = [torch.as_tensor(rng.standard_normal((d, r)).astype(np.float32).astype(np.float64)).cuda() for d, r in zip(dims, ranks)]
+    monkeypatch.setenv("TUCKER_TTMC_FIBERS", "0")
+    out = []
+    for chunk, x, u in ((32, vals, U), (1024, vals, U), (1024, vals.abs(), [a.abs() for a in U])):
+        monkeypatch.setenv("TUCKER_TTMC_CHUNK", str(chunk))
+        ctx = T.tucker_init(dims, coords, x, ranks, u)
+        assert T.tucker_mode_info(ctx, 0)["long_slices"] == (3000 if chunk == 32 else 0)
+        out.append(T.ttmc_mode(ctx, 0).double())
+        T.tucker_free(ctx)
+    assert ((out[0] - out[1]).abs() <= 2 * 600 * 2.0**-24 * out[2] * 1.001).all()
 
 
 def test_norms_of_cut_slices(monkeypatch):
