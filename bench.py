@@ -517,7 +517,7 @@ def run_mine(args):
             "config": {"workload": w.name, "dims": list(w.dims), "nnz": w.nnz, "nnz_coalesced": Zc,
                        "ranks": list(w.ranks), "l2": "flushed between timed steps (256 MiB write)",
                        "precision": "TTMc FP32 (FP32 products and sums); QRP: pivots and R from Y^T Y (exact "
-                                    "8-bit slices on the tensor cores, double-float sums, 2^-33), Q from the "
+                                    "8-bit slices on the tensor cores, double-float sums; decided within 2^-27), Q from the "
                                     "pivot columns in double-float with its orthogonality corrected (2e-14), "
                                     "stored in FP64; core "
                                     "on the tensor cores: Y (FP32) and U_N (FP64) cut into four exact 8-bit "

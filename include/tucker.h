@@ -54,8 +54,8 @@ typedef enum {
 /* Flags for tucker_init. */
 #define TUCKER_F_BF16_FACTORS 0x1u /* TTMc reads BF16 copies of the factors (FP32 accumulation); the
                                       faster option at order 3 and ranks 16 and 32.  At order 4 it is
-                                      the slower one (5M nonzeros, ranks 8^4: a sweep 3.67 ms, FP32
-                                      2.90 ms), at other ranks the time is that of FP32 */
+                                      the slower one (5M nonzeros, ranks 8^4: a sweep 3.54 ms, FP32
+                                      2.77 ms), at other ranks the time is that of FP32 */
 #define TUCKER_F_QRP_DIRECT 0x2u   /* fat Y_(n) (P_n > I_n): QRP on Y_(n) itself, not on Y Y^T */
 #define TUCKER_F_HOST_INPUT 0x4u   /* coords, vals and U0 given to tucker_init are host pointers */
 #define TUCKER_F_FIT_DEVICE 0x8u   /* hooi_iter writes the fit through a device pointer, no sync */
